@@ -1,7 +1,7 @@
 // rt_assemble.cu -- assembly of the operator on the GPU (Section 2, 2.1):
 //   * constants: Gauss-Legendre nodes, tetrahedron and triangle rules
-//   * entry kernels (warp per entry) for dense blocks, ACA rows/columns and
-//     arbitrary entry lists
+//   * entry kernels (warp per entry) for dense mode and arbitrary entry lists
+//     (rows and columns of the H-matrix build: rt_rows.cuh)
 //   * the emitter source Sbar^E
 //   * batched partially pivoted ACA with pivots shared by all kappa groups
 #include <algorithm>
@@ -17,6 +17,7 @@
 
 #include "rt_entry.cuh"
 #include "rt_internal.h"
+#include "rt_rows.h"
 
 namespace rt {
 
@@ -102,6 +103,12 @@ static void tri_rules(double* b, double* w)
         }
 }
 
+void quadrature_rules(double (&tet_b)[72], double (&tet_w)[18], double (&tri_b)[30], double (&tri_w)[10])
+{
+    tet_rules(tet_b, tet_w);
+    tri_rules(tri_b, tri_w);
+}
+
 int assemble_setup_constants(Operator& op, std::string& err)
 {
     std::vector<double> t, w;
@@ -113,29 +120,7 @@ int assemble_setup_constants(Operator& op, std::string& err)
         op.kp.gu32[g] = (float)u;
         op.kp.gw32[g] = (float)hw;
     }
-    // fixed rule tables: uploaded once per device (serialised across host threads)
-    static bool done[64] = {false};
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
-    int dev = 0;
-    RT_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 64 && done[dev]) return RT_OK;
-    double tb[18 * 4], tw[18];
-    float tbf[18 * 4], twf[18];
-    tet_rules(tb, tw);
-    for (int k = 0; k < 72; ++k) tbf[k] = (float)tb[k];
-    for (int k = 0; k < 18; ++k) twf[k] = (float)tw[k];
-    double rb[30], rw[10];
-    tri_rules(rb, rw);
-    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tet_b, tb, sizeof(tb)));
-    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tet_w, tw, sizeof(tw)));
-    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tet_bf, tbf, sizeof(tbf)));
-    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tet_wf, twf, sizeof(twf)));
-    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tri_b, rb, sizeof(rb)));
-    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tri_w, rw, sizeof(rw)));
-    RT_CUDA_TRY(cudaDeviceSynchronize());
-    if (dev < 64) done[dev] = true;
-    return RT_OK;
+    return upload_rules(err);
 }
 
 // ---------------------------------------------------------------------------
@@ -170,185 +155,6 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) entries_span_kernel(KernelP
 #pragma unroll
         for (int g = 0; g < MG; ++g)
             if (g < P.G && lane == (g & 31)) out[sp.base + g * sp.gs + ii * sp.is + jj * sp.js] = (OUT)acc[g];
-    }
-}
-
-// ACA rows (mode 0) / columns (mode 1) of the active far blocks.
-struct AcaActive {
-    int b;          // far block id
-    int row0, m, col0, n;
-    int64_t rbuf;   // offset of this block's [G][n] row buffer
-    int64_t cbuf;   // offset of this block's [G][m] column buffer
-    int64_t first_row, first_col;   // prefix of n (rows) and m (cols) over the active list
-    int64_t uoff, voff;             // pool offsets of this step's u [G][m] and v [G][n]
-    int64_t dot0;                   // first entry of this block's rank+1 dot products this step
-    int64_t first_chunk;            // prefix of ceil(m / kColRows) over the active list
-    int skip;       // set by the pivot kernel: zero row, no rank this step
-};
-
-__device__ __forceinline__ int find_active(const AcaActive* a, int na, int64_t e, int mode)
-{
-    int lo = 0, hi = na - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        int64_t f = mode == 0 ? a[mid].first_row : (mode == 1 ? a[mid].first_col : a[mid].first_chunk);
-        if (f <= e) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// ACA pivot columns: G_g[i, j*] for the rows i of an active block.  One CTA of
-// kColRows threads per chunk of kColRows rows.  The quadrature points of the
-// tetrahedra around the pivot vertex j* do not depend on the row, so each CTA
-// tabulates them once per batch of 32 tetrahedra in shared memory (position,
-// and vol * w_q * lambda_j(y) * kappa(y) / 4 pi for both rules) and every row
-// walks the table -- the sums of entry_warp, with each point's position,
-// kappa and hat-function weight computed once per chunk instead of per entry.
-constexpr int kColRows = 64;
-constexpr int kColTets = 32;
-
-// acc[g] += w exp(-c_g tau) over the groups; the factor c_g of Eq. 5 (the
-// group scale of the multi-frequency operator) multiplies the finished sums.
-// exp recurrence when c_g is arithmetic.
-template <int MG, bool XT = false>
-__device__ __forceinline__ void row_accumulate(const KernelParams& P, float (&acc)[MG], float w, float tau)
-{
-    if constexpr (XT) {
-        if (!(tau < INFINITY)) return;   // path through an opaque box
-    }
-    if (P.c_arith) {
-        float E = expf(-P.c0f * tau);
-        const float D = expf(-P.dcf * tau);
-#pragma unroll
-        for (int g = 0; g < MG; ++g) {
-            if (g < P.G) acc[g] += w * E;
-            E *= D;
-        }
-    } else {
-#pragma unroll
-        for (int g = 0; g < MG; ++g)
-            if (g < P.G) acc[g] += w * expf(-P.cf[g] * tau);
-    }
-}
-
-// add this thread's counts to the work counters (one atomic per warp and counter)
-__device__ __forceinline__ void count_work(const KernelParams& P, unsigned terms, unsigned depths)
-{
-    if (!P.work) return;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        terms += __shfl_xor_sync(0xffffffffu, terms, o);
-        depths += __shfl_xor_sync(0xffffffffu, depths, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(P.work, (unsigned long long)terms);
-        atomicAdd(P.work + 1, (unsigned long long)depths);
-    }
-}
-
-template <int MG, bool XT = false>
-__global__ void __launch_bounds__(kColRows) aca_col_kernel(KernelParams P, const AcaActive* __restrict__ act, int na,
-                                                           int64_t nchunks, const int* __restrict__ jstar,
-                                                           float* __restrict__ buf)
-{
-    __shared__ float4 s_pt[kColTets][18];   // rule rows 0-3: 4-point rule, 4-17: 14-point rule
-    __shared__ float4 s_cen[kColTets];      // centroid, 4 diam^2
-    const float inv4pi = (float)(1.0 / (4.0 * kPi));
-    for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-        const int ai = find_active(act, na, c, 2);
-        const AcaActive a = act[ai];
-        if (a.skip) continue;   // CTA-uniform
-        const int r0 = (int)(c - a.first_chunk) * kColRows;
-        const int j = a.col0 + jstar[a.b];
-        const int pos = r0 + threadIdx.x;
-        const bool row_ok = pos < a.m;
-        const int i = a.row0 + (row_ok ? pos : 0);
-        const Vec3<float> xi = load_xyz<float>(P, i);
-        Vec3<float> xb = xi;
-        if (P.has_wall) xb = mirror_point<float>(P, xi);
-        float acc[MG];
-#pragma unroll
-        for (int g = 0; g < MG; ++g) acc[g] = 0.f;
-        const int t0 = P.vt_ptr[j], t1 = P.vt_ptr[j + 1];
-        unsigned n_terms = 0, n_depths = 0;
-        for (int b0 = t0; b0 < t1; b0 += kColTets) {
-            const int nt = min(kColTets, t1 - b0);
-            __syncthreads();   // the previous batch's table is no longer read
-            for (int e = threadIdx.x; e < nt * 18; e += blockDim.x) {
-                const int t = e / 18, q = e - t * 18;
-                const int packed = P.vt_idx[b0 + t];
-                const int tet = packed >> 2, loc = packed & 3;
-                const int4 tv = P.tet[tet];
-                const Vec3<float> v0 = load_xyz<float>(P, tv.x), v1 = load_xyz<float>(P, tv.y),
-                                  v2 = load_xyz<float>(P, tv.z), v3 = load_xyz<float>(P, tv.w);
-                const float b0w = tet_b<float>(q, 0), b1 = tet_b<float>(q, 1), b2 = tet_b<float>(q, 2),
-                            b3 = tet_b<float>(q, 3);
-                Vec3<float> y;
-                y.x = b0w * v0.x + b1 * v1.x + b2 * v2.x + b3 * v3.x;
-                y.y = b0w * v0.y + b1 * v1.y + b2 * v2.y + b3 * v3.y;
-                y.z = b0w * v0.z + b1 * v1.z + b2 * v2.z + b3 * v3.z;
-                const float lam = loc == 0 ? b0w : (loc == 1 ? b1 : (loc == 2 ? b2 : b3));
-                const float w = P.tvol32[tet] * tet_w<float>(q) * lam * kappa_at<float, XT>(P, y.x, y.y, y.z) * inv4pi;
-                s_pt[t][q] = make_float4(y.x, y.y, y.z, w);
-                if (q == 0) {
-                    Vec3<float> cen;
-                    float diam, vol;
-                    load_tgeo<float>(P, tet, cen, diam, vol);
-                    s_cen[t] = make_float4(cen.x, cen.y, cen.z, 4.f * diam * diam);
-                }
-            }
-            __syncthreads();
-            if (row_ok) {
-                for (int t = 0; t < nt; ++t) {
-                    const float4 ce = s_cen[t];
-                    const Vec3<float> cen = {ce.x, ce.y, ce.z};
-                    const int nd = dist2<float>(xi, cen) < ce.w ? 14 : 4;
-                    const int nr = P.has_wall ? (dist2<float>(xb, cen) < ce.w ? 14 : 4) : 0;
-                    n_terms += nd + nr;
-                    n_depths += nd + 2 * nr;
-                    // direct points first, then the mirror-reflected ones: two
-                    // loops, so that lanes whose rules differ never run the
-                    // direct and the reflected branch at the same step
-                    const float4* pd = s_pt[t] + (nd == 14 ? 4 : 0);
-                    for (int q = 0; q < nd; ++q) {
-                        const float4 pt = pd[q];
-                        const Vec3<float> y = {pt.x, pt.y, pt.z};
-                        row_accumulate<MG, XT>(P, acc, pt.w / dist2<float>(xi, y), optical_depth<float, XT>(P, xi, y));
-                    }
-                    const float4* pr = s_pt[t] + (nr == 14 ? 4 : 0);
-                    for (int q = 0; q < nr; ++q) {
-                        const float4 pt = pr[q];
-                        const Vec3<float> y = {pt.x, pt.y, pt.z};
-                        const Vec3<float> xp = wall_point<float>(P, xb, y);
-                        const float tau = optical_depth<float, XT>(P, xi, xp) + optical_depth<float, XT>(P, xp, y);
-                        row_accumulate<MG, XT>(P, acc, (float)P.R0 * pt.w / dist2<float>(xb, y), tau);
-                    }
-                    if constexpr (XT) {   // further walls, corner paths
-                        for (int k = 0; k < P.n_extra; ++k) {
-                            Vec3<float> src;
-                            float sc;
-                            extra_term<float>(P, k, xi, src, sc);
-                            const int nx = dist2<float>(src, cen) < ce.w ? 14 : 4;
-                            n_terms += nx;
-                            n_depths += nx * (P.xkind[k] + 1);
-                            const float4* px = s_pt[t] + (nx == 14 ? 4 : 0);
-                            for (int q = 0; q < nx; ++q) {
-                                const float4 pt = px[q];
-                                const Vec3<float> y = {pt.x, pt.y, pt.z};
-                                row_accumulate<MG, XT>(P, acc, sc * pt.w / dist2<float>(src, y),
-                                                   extra_tau<float>(P, k, xi, src, y));
-                            }
-                        }
-                    }
-                }
-            }
-        }
-        if (row_ok) {
-#pragma unroll
-            for (int g = 0; g < MG; ++g)
-                if (g < P.G) buf[a.cbuf + (int64_t)g * a.m + pos] = acc[g] * P.cf[g];
-        }
-        count_work(P, n_terms, n_depths);
     }
 }
 
@@ -650,202 +456,16 @@ int assemble_source(Operator& op, cudaStream_t s, std::string& err)
     return RT_OK;
 }
 
-// ---------------------------------------------------------------------------
-// Row evaluation over a column cluster: G_g[i, j] for every column j of a
-// sub-cluster (at most kSubCols consecutive tree-order columns).  Each
-// tetrahedron touching the sub-cluster is visited once: every quadrature
-// point's kernel value feeds the (up to 4) hat functions of the tetrahedron's
-// vertices that lie in the sub-cluster -- the same sums as entry_warp, in a
-// different order, with each point evaluated once instead of once per vertex.
-// One CTA per (row, sub-cluster); the row segment accumulates in shared
-// memory [G][n] (float atomics, so the summation order is not fixed).
-// ---------------------------------------------------------------------------
-// threads of one row-over-cluster CTA: a (row, sub-cluster) item has a few
-// hundred tetrahedra, so 128 threads keep each thread busy on several of them
-// and let four CTAs per SM hide one another's end-of-item barrier
-constexpr int kRowThreads = 128;
-
-struct RowItem {
-    int b;            // ACA block (row = i + istar[b]) or -1 (row = i)
-    int i;
-    int col0, n;      // sub-cluster columns
-    int tet0, ntet;   // its tetrahedra in the sub-cluster tet list
-    int64_t out;      // output offset of (column col0, group 0)
-    int64_t gs, js;   // group and column strides of the output
-};
-
-// MG > 0: the four vertex sums of a tetrahedron accumulate in registers for
-// all groups and are flushed once per tetrahedron; MG == 0 (more than 32
-// groups): every point is added to shared memory directly.  Tetrahedra are
-// handed out through a shared counter so that the few tetrahedra near x_i
-// (14-point rules) do not hold up a fixed partition.
-template <int MG, bool XT = false>
-__global__ void __launch_bounds__(kRowThreads, MG <= 16 && !XT ? 4 : 2) row_cluster_kernel(KernelParams P, const RowItem* __restrict__ items,
-                                                          const int* __restrict__ sub_tets,
-                                                          const int* __restrict__ istar, float* __restrict__ out)
+void eval_tables_free(Operator& op)
 {
-    extern __shared__ float acc[];   // [G][n]
-    __shared__ int s_next;
-    const RowItem it = items[blockIdx.x];
-    const int i = it.b >= 0 ? it.i + istar[it.b] : it.i;
-    const int G = P.G, n = it.n;
-    for (int k = threadIdx.x; k < G * n; k += blockDim.x) acc[k] = 0.f;
-    if (threadIdx.x == 0) s_next = 0;
-    __syncthreads();
-    const Vec3<float> xi = load_xyz<float>(P, i);
-    Vec3<float> xb = xi;
-    if (P.has_wall) xb = mirror_point<float>(P, xi);
-    const float inv4pi = (float)(1.0 / (4.0 * kPi));
-    unsigned n_terms = 0, n_depths = 0;
-    for (;;) {
-        const int t = atomicAdd(&s_next, 1);
-        if (t >= it.ntet) break;
-        const int tet = sub_tets[it.tet0 + t];
-        const int4 tv = P.tet[tet];
-        const int jj[4] = {tv.x - it.col0, tv.y - it.col0, tv.z - it.col0, tv.w - it.col0};
-        const bool in0 = (unsigned)jj[0] < (unsigned)n, in1 = (unsigned)jj[1] < (unsigned)n,
-                   in2 = (unsigned)jj[2] < (unsigned)n, in3 = (unsigned)jj[3] < (unsigned)n;
-        const Vec3<float> v0 = load_xyz<float>(P, tv.x), v1 = load_xyz<float>(P, tv.y), v2 = load_xyz<float>(P, tv.z),
-                          v3 = load_xyz<float>(P, tv.w);
-        Vec3<float> cen;
-        float diam, vol;
-        load_tgeo<float>(P, tet, cen, diam, vol);
-        const float lim = 4.f * diam * diam;
-        const int nd = dist2<float>(xi, cen) < lim ? 14 : 4;
-        const int nr = P.has_wall ? (dist2<float>(xb, cen) < lim ? 14 : 4) : 0;
-        n_terms += nd + nr;
-        n_depths += nd + 2 * nr;
-        float a0[MG > 0 ? MG : 1], a1[MG > 0 ? MG : 1], a2[MG > 0 ? MG : 1], a3[MG > 0 ? MG : 1];
-        if constexpr (MG > 0) {
-#pragma unroll
-            for (int g = 0; g < MG; ++g) a0[g] = a1[g] = a2[g] = a3[g] = 0.f;
-        }
-        // Pass 0 visits the direct rule's points; when the reflected rule is
-        // the same one (nd == nr, the usual case away from the wall), the
-        // point, its weight and kappa(y) serve both terms.  Pass 1 visits the
-        // reflected rule's points only when the two rules differ.
-        const bool share = nd == nr;
-        for (int pass = 0; pass < 2; ++pass) {
-            const int nq = pass == 0 ? nd : (share ? 0 : nr);
-            const int base = (pass == 0 ? nd : nr) == 14 ? 4 : 0;
-            for (int q = 0; q < nq; ++q) {
-                const int row = base + q;
-                const float b0 = tet_b<float>(row, 0), b1 = tet_b<float>(row, 1), b2 = tet_b<float>(row, 2),
-                            b3 = tet_b<float>(row, 3);
-                Vec3<float> y;
-                y.x = b0 * v0.x + b1 * v1.x + b2 * v2.x + b3 * v3.x;
-                y.y = b0 * v0.y + b1 * v1.y + b2 * v2.y + b3 * v3.y;
-                y.z = b0 * v0.z + b1 * v1.z + b2 * v2.z + b3 * v3.z;
-                const float wq = vol * tet_w<float>(row) * kappa_at<float, XT>(P, y.x, y.y, y.z) * inv4pi;
-                auto accumulate = [&](float w, float tau) {
-                    if constexpr (XT) {
-                        if (!(tau < INFINITY)) return;   // path through an opaque box
-                    }
-                    if constexpr (MG > 0) {
-                        // c_g multiplies the sums when they are flushed
-                        const float w0 = w * b0, w1 = w * b1, w2 = w * b2, w3 = w * b3;
-                        auto add = [&](int g, float eg) {
-                            a0[g] += w0 * eg;
-                            a1[g] += w1 * eg;
-                            a2[g] += w2 * eg;
-                            a3[g] += w3 * eg;
-                        };
-                        if (P.c_arith) {
-                            // exp(-c_g tau) as exp(-c_0 tau) exp(-dc tau)^g: two SFU exponentials per point
-                            float E = expf(-P.c0f * tau);
-                            const float D = expf(-P.dcf * tau);
-#pragma unroll
-                            for (int g = 0; g < MG; ++g) {
-                                if (g < G) add(g, E);
-                                E *= D;
-                            }
-                        } else {
-#pragma unroll
-                            for (int g = 0; g < MG; ++g)
-                                if (g < G) add(g, expf(-P.cf[g] * tau));
-                        }
-                    } else {
-                        for (int g = 0; g < G; ++g) {
-                            const float cg = P.cf[g];
-                            const float val = w * cg * expf(-cg * tau);
-                            float* a = acc + g * n;
-                            if (in0) atomicAdd(a + jj[0], val * b0);
-                            if (in1) atomicAdd(a + jj[1], val * b1);
-                            if (in2) atomicAdd(a + jj[2], val * b2);
-                            if (in3) atomicAdd(a + jj[3], val * b3);
-                        }
-                    }
-                };
-                if (pass == 0) accumulate(wq / dist2<float>(xi, y), optical_depth<float, XT>(P, xi, y));
-                if (pass == 1 || share) {
-                    const Vec3<float> xp = wall_point<float>(P, xb, y);
-                    const float tau = optical_depth<float, XT>(P, xi, xp) + optical_depth<float, XT>(P, xp, y);
-                    accumulate((float)P.R0 * wq / dist2<float>(xb, y), tau);
-                }
-            }
-        }
-        if constexpr (XT) {
-            // further walls and corner paths, each with its own rule; the point
-            // value is split over the vertices as above
-            for (int k = 0; k < P.n_extra; ++k) {
-                Vec3<float> src;
-                float sc;
-                extra_term<float>(P, k, xi, src, sc);
-                const int nx = dist2<float>(src, cen) < lim ? 14 : 4;
-                n_terms += nx;
-                n_depths += nx * (P.xkind[k] + 1);
-                for (int q = 0; q < nx; ++q) {
-                    const int row = (nx == 14 ? 4 : 0) + q;
-                    const float b0 = tet_b<float>(row, 0), b1 = tet_b<float>(row, 1), b2 = tet_b<float>(row, 2),
-                                b3 = tet_b<float>(row, 3);
-                    const Vec3<float> y = {b0 * v0.x + b1 * v1.x + b2 * v2.x + b3 * v3.x,
-                                           b0 * v0.y + b1 * v1.y + b2 * v2.y + b3 * v3.y,
-                                           b0 * v0.z + b1 * v1.z + b2 * v2.z + b3 * v3.z};
-                    const float w = sc * vol * tet_w<float>(row) * kappa_at<float, XT>(P, y.x, y.y, y.z) * inv4pi /
-                                    dist2<float>(src, y);
-                    const float tau = extra_tau<float>(P, k, xi, src, y);
-                    if constexpr (MG > 0) {
-#pragma unroll
-                        for (int g = 0; g < MG; ++g)
-                            if (g < G) {
-                                const float val = w * expf(-P.cf[g] * tau);   // c_g at the flush
-                                a0[g] += val * b0;
-                                a1[g] += val * b1;
-                                a2[g] += val * b2;
-                                a3[g] += val * b3;
-                            }
-                    } else {
-                        for (int g = 0; g < G; ++g) {
-                            const float val = w * P.cf[g] * expf(-P.cf[g] * tau);
-                            float* a = acc + g * n;
-                            if (in0) atomicAdd(a + jj[0], val * b0);
-                            if (in1) atomicAdd(a + jj[1], val * b1);
-                            if (in2) atomicAdd(a + jj[2], val * b2);
-                            if (in3) atomicAdd(a + jj[3], val * b3);
-                        }
-                    }
-                }
-            }
-        }
-        if constexpr (MG > 0) {
-#pragma unroll
-            for (int g = 0; g < MG; ++g)
-                if (g < G) {
-                    float* a = acc + g * n;
-                    const float cg = P.cf[g];
-                    if (in0) atomicAdd(a + jj[0], a0[g] * cg);
-                    if (in1) atomicAdd(a + jj[1], a1[g] * cg);
-                    if (in2) atomicAdd(a + jj[2], a2[g] * cg);
-                    if (in3) atomicAdd(a + jj[3], a3[g] * cg);
-                }
-        }
-    }
-    count_work(P, n_terms, n_depths);
-    __syncthreads();
-    for (int k = threadIdx.x; k < G * n; k += blockDim.x) {
-        const int g = k / n, j = k - g * n;
-        out[it.out + g * it.gs + j * it.js] = acc[k];
-    }
+    for (void* p : op.eval_tables) cudaFreeAsync(p, op.stream);
+    op.eval_tables.clear();
+    op.eval_bytes = 0;
+    op.d_sub_tets = nullptr;
+    op.d_subs = nullptr;
+    op.d_pass_ref = nullptr;
+    op.d_pass_run = nullptr;
+    op.kp.pxyz = op.kp.pcos = op.kp.tcen = op.kp.tpt = op.kp.tcos = nullptr;
 }
 
 // sub-clusters of every column cluster and the tetrahedra touching each
@@ -903,28 +523,11 @@ int prepare_row_eval(Operator& op, std::string& err)
         }
         op.sub_of_cluster_ptr[c + 1] = (int)op.sub_of_cluster.size();
     }
-    int rc = dev_alloc(op, &op.d_sub_tets, tets.size(), err);
-    if (rc) return rc;
-    if ((rc = upload_async(op, op.d_sub_tets, tets.data(), tets.size(), err))) return rc;
-    static bool attr_set[64] = {false};
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 64 && !attr_set[dev]) {
-        const int bytes = (int)(kMaxGroups * kSubCols * sizeof(float));
-        RT_CUDA_TRY(cudaFuncSetAttribute(row_cluster_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-        RT_CUDA_TRY(cudaFuncSetAttribute(row_cluster_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-        RT_CUDA_TRY(cudaFuncSetAttribute(row_cluster_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-        RT_CUDA_TRY(cudaFuncSetAttribute(row_cluster_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-        RT_CUDA_TRY(cudaFuncSetAttribute(row_cluster_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-        RT_CUDA_TRY(cudaFuncSetAttribute(row_cluster_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-        RT_CUDA_TRY(cudaFuncSetAttribute(row_cluster_kernel<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-        RT_CUDA_TRY(cudaFuncSetAttribute(row_cluster_kernel<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-        attr_set[dev] = true;
-    }
-    return RT_OK;
+    return RT_EVALUATOR(op, tables(op, tets, err));
 }
+
+// most rows of one item: the sums of all its rows take at most 32 KB
+static int rows_per_item(int mg, int n) { return std::max(1, std::min(8, 32768 / (4 * mg * n))); }
 
 static int launch_rows(Operator& op, const std::vector<RowItem>& items, const int* istar, float* out, cudaStream_t s,
                        std::string& err)
@@ -933,23 +536,13 @@ static int launch_rows(Operator& op, const std::vector<RowItem>& items, const in
     RowItem* d = nullptr;
     RT_CUDA_TRY(cudaMallocAsync((void**)&d, sizeof(RowItem) * items.size(), s));
     RT_CUDA_TRY(cudaMemcpyAsync(d, items.data(), sizeof(RowItem) * items.size(), cudaMemcpyHostToDevice, s));
-    int maxn = 0;
-    for (const RowItem& it : items) maxn = std::max(maxn, it.n);
-    const size_t smem = (size_t)op.G * maxn * sizeof(float);
+    int sums = 0;
+    for (const RowItem& it : items) sums = std::max(sums, it.nrow * op.sub_size[it.sub]);
     for (size_t k0 = 0; k0 < items.size(); k0 += (size_t)1 << 30) {
-        const int cnt = (int)std::min<size_t>(items.size() - k0, (size_t)1 << 30);
-        const int G = op.G;
-        if (op.kp.ext) {   // further walls, corner paths, a kappa grid or opaque boxes
-            if (G <= 16) row_cluster_kernel<16, true><<<cnt, kRowThreads, smem, s>>>(op.kp, d + k0, op.d_sub_tets, istar, out);
-            else row_cluster_kernel<0, true><<<cnt, kRowThreads, smem, s>>>(op.kp, d + k0, op.d_sub_tets, istar, out);
-        } else if (G <= 1) row_cluster_kernel<1><<<cnt, kRowThreads, smem, s>>>(op.kp, d + k0, op.d_sub_tets, istar, out);
-        else if (G <= 4) row_cluster_kernel<4><<<cnt, kRowThreads, smem, s>>>(op.kp, d + k0, op.d_sub_tets, istar, out);
-        else if (G <= 8) row_cluster_kernel<8><<<cnt, kRowThreads, smem, s>>>(op.kp, d + k0, op.d_sub_tets, istar, out);
-        else if (G <= 16) row_cluster_kernel<16><<<cnt, kRowThreads, smem, s>>>(op.kp, d + k0, op.d_sub_tets, istar, out);
-        else if (G <= 32) row_cluster_kernel<32><<<cnt, kRowThreads, smem, s>>>(op.kp, d + k0, op.d_sub_tets, istar, out);
-        else row_cluster_kernel<0><<<cnt, kRowThreads, smem, s>>>(op.kp, d + k0, op.d_sub_tets, istar, out);
+        const int n = (int)std::min<size_t>(items.size() - k0, (size_t)1 << 30);
+        const int rc = RT_EVALUATOR(op, rows(op, d + k0, n, sums, istar, out, s, err));
+        if (rc) return rc;
     }
-    RT_CUDA_TRY(cudaGetLastError());
     RT_CUDA_TRY(cudaFreeAsync(d, s));
     return RT_OK;
 }
@@ -1001,6 +594,17 @@ struct AcaDev {
     double* dots;       // per step: [dot0 + l][G][2]  (u_l.u, v_l.v), l = rank -> (|u|^2, |v|^2)
     float* pool;
 };
+
+__device__ __forceinline__ int find_active(const AcaActive* a, int na, int64_t e, int mode)
+{
+    int lo = 0, hi = na - 1;
+    while (lo < hi) {
+        int mid = (lo + hi + 1) >> 1;
+        const int64_t f = mode == 0 ? a[mid].first_row : a[mid].first_col;
+        if (f <= e) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
 
 // residual row: R_g[jj] -= sum_l u_{g,l}[i*] v_{g,l}[jj]; row key = argmax score.
 __global__ void aca_row_residual(AcaDev D, const AcaActive* act, int na, int64_t total, float* buf)
@@ -1304,7 +908,7 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
     std::vector<void*> tmp;   // freed at the end
     int64_t scratch = 0;      // bytes of ACA scratch held now (tmp, pool, dot lists)
     auto note_peak = [&](int64_t extra) {
-        op.info.peak_bytes = std::max<int64_t>(op.info.peak_bytes, op.info.device_bytes + scratch + extra);
+        op.info.peak_bytes = std::max<int64_t>(op.info.peak_bytes, op.info.device_bytes + op.eval_bytes + scratch + extra);
     };
     auto talloc = [&](void** p, size_t bytes) -> int {
         cudaError_t e = cudaMallocAsync(p, bytes ? bytes : 1, s);
@@ -1511,7 +1115,7 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                     a.dot0 = ndot;
                     ndot += h_rank[b] + 1;
                     a.first_chunk = nchunk;
-                    nchunk += (a.m + kColRows - 1) / kColRows;
+                    nchunk += col_chunks(a.m);
                     fr += a.n;
                     fc += a.m;
                     bufr += (int64_t)G * a.n;
@@ -1530,10 +1134,8 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                             RowItem it{};
                             it.b = a.b;
                             it.i = fb.row0;
-                            it.col0 = op.sub_start[sb];
-                            it.n = op.sub_size[sb];
-                            it.tet0 = op.sub_tet_ptr[sb];
-                            it.ntet = op.sub_tet_ptr[sb + 1] - op.sub_tet_ptr[sb];
+                            it.nrow = 1;
+                            it.sub = sb;
                             it.out = a.rbuf + (op.sub_start[sb] - fb.col0);
                             it.gs = fb.n;
                             it.js = 1;
@@ -1552,15 +1154,10 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                 // 2. pivot columns: one CTA per 64-row chunk, the column's quadrature
                 // points tabulated once per chunk
                 {
-                    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(nchunk, (int64_t)sms * 32));
-#define RT_LAUNCH_ACAC(MG, XT) \
-    aca_col_kernel<MG, XT><<<grid, kColRows, 0, s>>>(op.kp, d_act, na, nchunk, D.jstar, colbuf)
-#define RT_LAUNCH_ACAC1(MG) RT_LAUNCH_ACAC(MG, false)
-                    if (op.kp.ext) RT_DISPATCH_MG_XT(G, RT_LAUNCH_ACAC);
-                    else RT_DISPATCH_MG(G, RT_LAUNCH_ACAC1);
-#undef RT_LAUNCH_ACAC1
-#undef RT_LAUNCH_ACAC
-                    RT_CUDA_TRY(cudaGetLastError());
+                    if ((rc = RT_EVALUATOR(op, columns(op, d_act, na, nchunk, D.jstar, colbuf, s, err)))) {
+                        cleanup();
+                        return rc;
+                    }
                 }
                 const int eg_c = (int)std::min<int64_t>((fc + 255) / 256, (int64_t)sms * 32);
                 aca_col_residual<<<std::max(1, eg_c), 256, 0, s>>>(D, d_act, na, fc, colbuf);
@@ -1722,21 +1319,21 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
             const FarBlock& fb = op.dense_blocks[k];
             for (int c = op.dense_chunk_ptr[k]; c < op.dense_chunk_ptr[k + 1]; ++c) {
                 const Chunk& ch = op.dense_chunks[c];
-                for (int ii = 0; ii < ch.m; ++ii)
-                    for (int e = op.sub_of_cluster_ptr[fb.sc]; e < op.sub_of_cluster_ptr[fb.sc + 1]; ++e) {
-                        const int sb = op.sub_of_cluster[e];
+                for (int e = op.sub_of_cluster_ptr[fb.sc]; e < op.sub_of_cluster_ptr[fb.sc + 1]; ++e) {
+                    const int sb = op.sub_of_cluster[e];
+                    const int rows = rows_per_item(group_chunk(op), op.sub_size[sb]);
+                    for (int ii = 0; ii < ch.m; ii += rows) {
                         RowItem it{};
                         it.b = -1;
                         it.i = fb.row0 + ch.rbeg + ii;
-                        it.col0 = op.sub_start[sb];
-                        it.n = op.sub_size[sb];
-                        it.tet0 = op.sub_tet_ptr[sb];
-                        it.ntet = op.sub_tet_ptr[sb + 1] - op.sub_tet_ptr[sb];
+                        it.nrow = std::min(rows, ch.m - ii);
+                        it.sub = sb;
                         it.out = op.dense_off[k] + ch.off + ii + (int64_t)(op.sub_start[sb] - fb.col0) * ch.m8;
                         it.gs = (int64_t)fb.n * ch.m8;
                         it.js = ch.m8;
                         ritems.push_back(it);
                     }
+                }
             }
         }
         if ((rc = launch_rows(op, ritems, nullptr, op.d_near, s, err))) return rc;

@@ -218,6 +218,55 @@ int group_channels(rt::Operator& op, const rt_freqs& Fq, int bins, std::string& 
     return RT_OK;
 }
 
+// Whether the phase evaluator (rt_phase.cuh) serves the problem, and its
+// parameters: no further walls, grid or boxes; the first wall, if any, normal
+// to an axis with the whole mesh on its inner side; for the sin-product kappa
+// also the closed form of the Gauss sums on every path (the domain and its
+// shadow on the wall in a box of side sum <= 3).  The size limits keep r^2
+// inside the normal FP32 range.
+void phase_setup(rt::Operator& op, const std::vector<double>& xyz)
+{
+    rt::KernelParams& kp = op.kp;
+    kp.evaluator = kp.ext ? rt::EV_GENERAL : rt::EV_PLAIN;
+    kp.axis[0] = 0;
+    kp.axis[1] = 1;
+    kp.axis[2] = 2;
+    kp.wc0 = kp.wc0x2 = kp.wcos2 = 0.f;
+    kp.amp8pi = (float)(kp.amp / (8.0 * rt::kPi));
+    if (kp.ext) return;
+    double lo[3], hi[3];
+    for (int d = 0; d < 3; ++d) lo[d] = hi[d] = xyz[d];
+    for (size_t k = 3; k < xyz.size(); k += 3)
+        for (int d = 0; d < 3; ++d) {
+            lo[d] = std::min(lo[d], xyz[k + d]);
+            hi[d] = std::max(hi[d], xyz[k + d]);
+        }
+    double mag = 0.0;
+    for (int d = 0; d < 3; ++d) mag = std::max({mag, std::fabs(lo[d]), std::fabs(hi[d])});
+    if (kp.has_wall) {
+        int ax = -1;
+        for (int d = 0; d < 3; ++d)
+            if (std::fabs(kp.wn[d]) == 1.0) ax = d;
+        if (ax < 0) return;
+        const double c0 = kp.wp[ax];
+        if (kp.wn[ax] > 0.0 ? hi[ax] > c0 : lo[ax] < c0) return;
+        lo[ax] = std::min(lo[ax], c0);
+        hi[ax] = std::max(hi[ax], c0);
+        mag = std::max(mag, std::fabs(c0));
+        kp.axis[0] = ax == 0 ? 1 : 0;
+        kp.axis[1] = ax == 2 ? 1 : 2;
+        kp.axis[2] = ax;
+        kp.wc0 = (float)c0;
+        kp.wc0x2 = (float)(2.0 * c0);
+        kp.wcos2 = (float)(2.0 * std::cos(2.0 * rt::kPi * c0));
+    }
+    double size = 0.0;
+    for (int d = 0; d < 3; ++d) size += hi[d] - lo[d];
+    if (!(size < 1e15 && mag < 1e15 && op.min_diam > 1e-15)) return;
+    if (kp.sinprod && (!kp.line_closed || size > 3.0 || mag > 1e4)) return;
+    kp.evaluator = rt::EV_PHASE;
+}
+
 int build(rt::Operator& op, const rt_problem* P, const rt_hparams* H, cudaStream_t s, std::string& err,
           rt::Plan* pre)
 {
@@ -316,6 +365,7 @@ int build(rt::Operator& op, const rt_problem* P, const rt_hparams* H, cudaStream
         tg32[k] = make_float4((float)cen[0], (float)cen[1], (float)cen[2], (float)dm);
         tv64[k] = vol;
         tv32[k] = (float)vol;
+        op.min_diam = std::min(op.min_diam, dm);
         for (int d = 0; d < 4; ++d) cnt[a[d] + 1]++;
     }
     for (int64_t v = 0; v < N; ++v) cnt[v + 1] += cnt[v];
@@ -445,6 +495,40 @@ int build(rt::Operator& op, const rt_problem* P, const rt_hparams* H, cudaStream
     }
     kp.ngauss = op.ngauss;
     kp.line_closed = (H->line_eval == RT_LINE_CLOSED && op.ngauss >= 16) ? 1 : 0;
+    kp.sinprod = kp.kappa_kind == RT_KAPPA_SINPROD ? 1 : 0;
+    kp.R0f = (float)kp.R0;
+    for (int d = 0; d < 3; ++d) {
+        kp.wpf[d] = (float)kp.wp[d];
+        kp.wnf[d] = (float)kp.wn[d];
+    }
+    for (int w = 0; w < P->n_walls; ++w) {
+        for (int d = 0; d < 3; ++d) {
+            kp.wpsf[w][d] = (float)kp.wps[w][d];
+            kp.wnsf[w][d] = (float)kp.wns[w][d];
+        }
+        kp.wRf[w] = (float)kp.wR[w];
+    }
+    if (kp.kappa_kind == RT_KAPPA_GRID)
+        for (int d = 0; d < 3; ++d) {
+            kp.glof[d] = (float)kp.glo[d];
+            kp.ghif[d] = (float)kp.ghi[d];
+            kp.ghf[d] = (kp.ghif[d] - kp.glof[d]) / (float)kp.gdims[d];
+        }
+    for (int o = 0; o < kp.n_obst; ++o)
+        for (int d = 0; d < 3; ++d) {
+            kp.olof[o][d] = (float)kp.olo[o][d];
+            kp.ohif[o][d] = (float)kp.ohi[o][d];
+        }
+    const double log2e = 1.4426950408889634;
+    const double dl = -log2e * (op.G > 1 ? op.gc[1] - op.gc[0] : 0.0);
+    kp.dcl = (float)dl;
+    kp.dclo = (float)(dl - kp.dcl);
+    for (int g = 0; g < op.G; ++g) {
+        const double l = -log2e * op.gc[g];
+        kp.cl[g] = (float)l;
+        kp.clo[g] = (float)(l - kp.cl[g]);
+    }
+    phase_setup(op, xyz64);
     kp.xyz32 = op.d_xyz32;
     kp.xyz64 = op.d_xyz64;
     kp.tet = op.d_tet;
@@ -476,6 +560,7 @@ int build(rt::Operator& op, const rt_problem* P, const rt_hparams* H, cudaStream
     } else {
         if ((rc = prepare_row_eval(op, err))) return rc;
         if ((rc = assemble_hmatrix(op, s, err))) return rc;
+        eval_tables_free(op);
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -544,6 +629,8 @@ void operator_release(Operator& op, cudaStream_t s)
     for (void* p : op.allocations)
         if (p) cudaFreeAsync(p, s);
     op.allocations.clear();
+    for (void* p : op.eval_tables) cudaFreeAsync(p, s);   // a build that failed midway
+    op.eval_tables.clear();
     if (op.far_buf.base || op.far_lo_buf.base) {
         // unmapping is not stream ordered: wait for the work queued on s
         cudaStreamSynchronize(s);

@@ -26,19 +26,46 @@
 // (kappa_nu = c_g kappa(x) => tau_g = c_g tau).
 #pragma once
 
+#include <mutex>
+
 #include "rt_internal.h"
 
 namespace rt {
 
 // Tetrahedron and triangle rules as barycentric coordinates, set from the
-// host once per device.  (The Gauss nodes live in KernelParams.)  This header
-// is included by one translation unit only.
-__constant__ double c_tet_b[18 * 4];  // rows 0..3: 4-point rule, rows 4..17: 14-point rule
-__constant__ double c_tet_w[18];
-__constant__ float c_tet_bf[18 * 4];
-__constant__ float c_tet_wf[18];
-__constant__ double c_tri_b[10 * 3];  // rows 0..2: 3-point rule, rows 3..9: 7-point rule
-__constant__ double c_tri_w[10];
+// host once per device.  (The Gauss nodes live in KernelParams.)  Every
+// translation unit that includes this header has its own copy.
+static __constant__ double c_tet_b[18 * 4];  // rows 0..3: 4-point rule, rows 4..17: 14-point rule
+static __constant__ double c_tet_w[18];
+static __constant__ float c_tet_bf[18 * 4];
+static __constant__ float c_tet_wf[18];
+static __constant__ double c_tri_b[10 * 3];  // rows 0..2: 3-point rule, rows 3..9: 7-point rule
+static __constant__ double c_tri_w[10];
+
+// this unit's tables, uploaded once per device (serialised across host threads)
+static int upload_rules(std::string& err)
+{
+    static bool done[64] = {false};
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    int dev = 0;
+    RT_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 64 && done[dev]) return RT_OK;
+    double tb[72], tw[18], rb[30], rw[10];
+    float tbf[72], twf[18];
+    quadrature_rules(tb, tw, rb, rw);
+    for (int k = 0; k < 72; ++k) tbf[k] = (float)tb[k];
+    for (int k = 0; k < 18; ++k) twf[k] = (float)tw[k];
+    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tet_b, tb, sizeof(tb)));
+    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tet_w, tw, sizeof(tw)));
+    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tet_bf, tbf, sizeof(tbf)));
+    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tet_wf, twf, sizeof(twf)));
+    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tri_b, rb, sizeof(rb)));
+    RT_CUDA_TRY(cudaMemcpyToSymbol(c_tri_w, rw, sizeof(rw)));
+    RT_CUDA_TRY(cudaDeviceSynchronize());
+    if (dev < 64) done[dev] = true;
+    return RT_OK;
+}
 
 template <class R>
 struct Vec3 {
@@ -192,6 +219,15 @@ __device__ __forceinline__ int grid_cell(const KernelParams& P, int d, R x)
     return (int)floor(u);
 }
 
+template <>
+__device__ __forceinline__ int grid_cell<float>(const KernelParams& P, int d, float x)
+{
+    const float n = (float)P.gdims[d];
+    float u = (x - P.glof[d]) / (P.ghif[d] - P.glof[d]) * n;
+    u = u < 0.f ? 0.f : (u > n - 0.5f ? n - 0.5f : u);
+    return (int)floorf(u);
+}
+
 template <class R>
 __device__ __forceinline__ R grid_kappa(const KernelParams& P, R x, R y, R z)
 {
@@ -339,6 +375,95 @@ __device__ bool path_blocked(const KernelParams& P, const Vec3<R>& a, const Vec3
     return false;
 }
 
+// The FP32 forms of grid_depth and path_blocked for one segment: the bounds as
+// FP32 parameters (an FP64 parameter converted inside the walk goes through the
+// FP64 unit, 1/64 of the FP32 rate) and one reciprocal per axis and segment
+// that every plane crossing and slab test multiplies with, where the general
+// forms divide.  Same planes, cells, order and tolerance.
+struct SegmentF {
+    float A[3], D[3], inv[3];
+};
+__device__ __forceinline__ SegmentF make_segment(const Vec3<float>& a, const Vec3<float>& b)
+{
+    SegmentF s = {{a.x, a.y, a.z}, {b.x - a.x, b.y - a.y, b.z - a.z}, {}};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) s.inv[d] = 1.f / s.D[d];
+    return s;
+}
+
+__device__ __forceinline__ bool segment_blocked(const KernelParams& P, const SegmentF& s)
+{
+    for (int o = 0; o < P.n_obst; ++o) {
+        float t0 = 0.f, t1 = 1.f;
+        bool inside = true;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float lo = P.olof[o][d], hi = P.ohif[o][d];
+            const float ta = (lo - s.A[d]) * s.inv[d], tb = (hi - s.A[d]) * s.inv[d];
+            const bool flat = s.D[d] == 0.f;
+            inside = inside && (!flat || (s.A[d] > lo && s.A[d] < hi));
+            t0 = flat ? t0 : fmaxf(t0, fminf(ta, tb));
+            t1 = flat ? t1 : fminf(t1, fmaxf(ta, tb));
+        }
+        if (inside && t1 - t0 > 1e-6f) return true;
+    }
+    return false;
+}
+
+__device__ __forceinline__ float segment_grid_depth(const KernelParams& P, const SegmentF& s)
+{
+    float tn[3];
+    int m[3], last[3], step[3], idx = 0, stride = 1;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int n = P.gdims[d];
+        const float lo = P.glof[d], h = P.ghf[d];
+        const bool up = s.D[d] > 0.f;
+        int cell;
+        tn[d] = 2.f;
+        m[d] = 0;
+        last[d] = up ? n - 1 : 1;
+        step[d] = up ? stride : -stride;
+        if (s.D[d] != 0.f) {
+            const float u = (s.A[d] - lo) / h;
+            const float uc = fminf(fmaxf(u, -1.f), (float)(n + 1));
+            m[d] = up ? max((int)floorf(uc) + 1, 1) : min((int)ceilf(uc) - 1, n - 1);
+            // first plane strictly ahead of a (rounding may put the first guess behind)
+            for (int it = 0; it < 3; ++it) {
+                if (m[d] < 1 || m[d] > n - 1 || (fmaf((float)m[d], h, lo) - s.A[d]) * s.inv[d] > 0.f) break;
+                m[d] += up ? 1 : -1;
+            }
+            if (m[d] >= 1 && m[d] <= n - 1) tn[d] = (fmaf((float)m[d], h, lo) - s.A[d]) * s.inv[d];
+            cell = min(max(up ? m[d] - 1 : m[d], 0), n - 1);
+        } else {
+            cell = grid_cell<float>(P, d, s.A[d]);
+        }
+        idx += cell * stride;
+        stride *= n;
+    }
+    float sum = 0.f, t0 = 0.f;
+    const int max_steps = P.gdims[0] + P.gdims[1] + P.gdims[2] + 4;
+    for (int k = 0; k < max_steps; ++k) {
+        const float v = __ldg(P.kgrid32 + idx);
+        const float tm = fminf(fminf(tn[0], tn[1]), tn[2]);
+        const float t1 = fminf(tm, 1.f);
+        if (t1 > t0) {
+            sum = fmaf(v, t1 - t0, sum);
+            t0 = t1;
+        }
+        if (t1 >= 1.f) break;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (tn[d] == t1) {
+                idx += step[d];
+                const bool end = m[d] == last[d];
+                m[d] += step[d] > 0 ? 1 : -1;
+                tn[d] = end ? 2.f : (fmaf((float)m[d], P.ghf[d], P.glof[d]) - s.A[d]) * s.inv[d];
+            }
+    }
+    return sqrtf(s.D[0] * s.D[0] + s.D[1] * s.D[1] + s.D[2] * s.D[2]) * sum;
+}
+
 // int_[a,b] kappa = |b-a| sum_g (w_g/2) kappa(a + u_g (b-a)).  For constant
 // kappa the Gauss sum equals kappa |b-a| exactly (weights sum to 1).  The
 // general instances (XT) also handle the opaque boxes (+infinity) and the
@@ -346,7 +471,13 @@ __device__ bool path_blocked(const KernelParams& P, const Vec3<R>& a, const Vec3
 template <class R, bool XT = false>
 __device__ __forceinline__ R optical_depth(const KernelParams& P, const Vec3<R>& a, const Vec3<R>& b)
 {
-    if constexpr (XT) {
+    if constexpr (XT && sizeof(R) == 4) {
+        if (P.n_obst > 0 || P.kappa_kind == RT_KAPPA_GRID) {
+            const SegmentF s = make_segment(a, b);
+            if (segment_blocked(P, s)) return INFINITY;
+            if (P.kappa_kind == RT_KAPPA_GRID) return segment_grid_depth(P, s);
+        }
+    } else if constexpr (XT) {
         if (P.n_obst > 0 && path_blocked<R>(P, a, b)) return R(INFINITY);
         if (P.kappa_kind == RT_KAPPA_GRID) return grid_depth<R>(P, a, b);
     }
@@ -371,6 +502,13 @@ __device__ __forceinline__ Vec3<R> mirror_point(const KernelParams& P, const Vec
     return {x.x - R(2) * s * R(P.wn[0]), x.y - R(2) * s * R(P.wn[1]), x.z - R(2) * s * R(P.wn[2])};
 }
 
+template <>
+__device__ __forceinline__ Vec3<float> mirror_point<float>(const KernelParams& P, const Vec3<float>& x)
+{
+    const float s = (x.x - P.wpf[0]) * P.wnf[0] + (x.y - P.wpf[1]) * P.wnf[1] + (x.z - P.wpf[2]) * P.wnf[2];
+    return {x.x - 2.f * s * P.wnf[0], x.y - 2.f * s * P.wnf[1], x.z - 2.f * s * P.wnf[2]};
+}
+
 // x' on the wall plane along [xbar, y]
 template <class R>
 __device__ __forceinline__ Vec3<R> wall_point(const KernelParams& P, const Vec3<R>& xb, const Vec3<R>& y)
@@ -382,6 +520,16 @@ __device__ __forceinline__ Vec3<R> wall_point(const KernelParams& P, const Vec3<
     return {xb.x + t * (y.x - xb.x), xb.y + t * (y.y - xb.y), xb.z + t * (y.z - xb.z)};
 }
 
+template <>
+__device__ __forceinline__ Vec3<float> wall_point<float>(const KernelParams& P, const Vec3<float>& xb, const Vec3<float>& y)
+{
+    const float sb = (xb.x - P.wpf[0]) * P.wnf[0] + (xb.y - P.wpf[1]) * P.wnf[1] + (xb.z - P.wpf[2]) * P.wnf[2];
+    const float sy = (y.x - P.wpf[0]) * P.wnf[0] + (y.y - P.wpf[1]) * P.wnf[1] + (y.z - P.wpf[2]) * P.wnf[2];
+    const float den = sb - sy;
+    const float t = den > 0.f ? sb / den : 0.f;
+    return {xb.x + t * (y.x - xb.x), xb.y + t * (y.y - xb.y), xb.z + t * (y.z - xb.z)};
+}
+
 // ---- further reflected terms (several walls, corner paths) -------------------
 template <class R>
 __device__ __forceinline__ R wall_side(const KernelParams& P, int w, const Vec3<R>& x)
@@ -390,11 +538,25 @@ __device__ __forceinline__ R wall_side(const KernelParams& P, int w, const Vec3<
            (x.z - R(P.wps[w][2])) * R(P.wns[w][2]);
 }
 
+template <>
+__device__ __forceinline__ float wall_side<float>(const KernelParams& P, int w, const Vec3<float>& x)
+{
+    return (x.x - P.wpsf[w][0]) * P.wnsf[w][0] + (x.y - P.wpsf[w][1]) * P.wnsf[w][1] + (x.z - P.wpsf[w][2]) * P.wnsf[w][2];
+}
+template <class R>
+__device__ __forceinline__ R wall_n(const KernelParams& P, int w, int d) { return R(P.wns[w][d]); }
+template <>
+__device__ __forceinline__ float wall_n<float>(const KernelParams& P, int w, int d) { return P.wnsf[w][d]; }
+template <class R>
+__device__ __forceinline__ R wall_R(const KernelParams& P, int w) { return R(P.wR[w]); }
+template <>
+__device__ __forceinline__ float wall_R<float>(const KernelParams& P, int w) { return P.wRf[w]; }
+
 template <class R>
 __device__ __forceinline__ Vec3<R> mirror_w(const KernelParams& P, int w, const Vec3<R>& x)
 {
     const R s = wall_side<R>(P, w, x);
-    return {x.x - R(2) * s * R(P.wns[w][0]), x.y - R(2) * s * R(P.wns[w][1]), x.z - R(2) * s * R(P.wns[w][2])};
+    return {x.x - R(2) * s * wall_n<R>(P, w, 0), x.y - R(2) * s * wall_n<R>(P, w, 1), x.z - R(2) * s * wall_n<R>(P, w, 2)};
 }
 
 // source point (the image of x) and weight of extra term k
@@ -403,10 +565,10 @@ __device__ __forceinline__ void extra_term(const KernelParams& P, int k, const V
 {
     const int a = P.xa[k];
     src = mirror_w<R>(P, a, x);
-    scale = R(P.wR[a]);
+    scale = wall_R<R>(P, a);
     if (P.xkind[k] == 2) {
         src = mirror_w<R>(P, P.xb[k], src);
-        scale *= R(P.wR[P.xb[k]]);
+        scale *= wall_R<R>(P, P.xb[k]);
     }
 }
 

@@ -29,6 +29,11 @@ constexpr int kMaxXTerms = 5;    // reflected terms beyond the first wall's: 2 w
 constexpr int kMaxObst = 4;      // opaque boxes per problem
 constexpr int kMaxGauss = 32;
 constexpr int kSubCols = 256;   // columns per sub-cluster in row evaluations
+
+// How the FP32 rows and columns evaluate a kernel value: phase tables
+// (rt_phase.cuh); optical_depth with one wall or none (oblique walls, node
+// sums); every term and medium.
+enum { EV_PHASE = 0, EV_PLAIN = 1, EV_GENERAL = 2 };
 constexpr double kPi = 3.14159265358979323846;
 
 struct alignas(16) dbl4 {
@@ -88,6 +93,24 @@ struct KernelParams {
     // assembly work counters (may be null): [0] kernel terms evaluated (one direct or
     // one reflected value e^{-c tau} / r^2 at a point pair), [1] optical depths
     unsigned long long* work;
+    // rows and columns of G in FP32 (rt_rows.cuh): tables per tetrahedron and point
+    // of the 4-point rule, and for the phase evaluator (rt_phase.cuh) permuted
+    // coordinates (p, q, c: the first wall's axis last) and phase cosines
+    int evaluator;      // EV_PHASE, EV_PLAIN or EV_GENERAL (rt_rows.cuh)
+    int sinprod;        // kappa_kind == RT_KAPPA_SINPROD
+    int axis[3];        // p, q, c as coordinate indices
+    float wc0, wc0x2, wcos2;   // wall position C0 along c, 2 C0, 2 cos(2 pi C0)
+    float R0f, amp8pi;  // R0; amp / (8 pi)
+    float wpf[3], wnf[3];      // the first wall's point and normal
+    // FP32 copies for the general FP32 kernels
+    float wpsf[kMaxWalls][3], wnsf[kMaxWalls][3], wRf[kMaxWalls];
+    float glof[3], ghif[3], ghf[3];   // grid box and cell sizes
+    float olof[kMaxObst][3], ohif[kMaxObst][3];
+    float dcl, dclo;           // -dc log2(e), -c_g log2(e): FP32 value and remainder
+    float cl[kMaxGroups], clo[kMaxGroups];
+    const float4 *pxyz, *pcos; // [N] permuted coordinates, cosines
+    const float4* tcen;        // [T] centroid, (2 diameters)^2
+    const float4 *tpt, *tcos;  // [4][T] point and weight, cosines
 };
 
 // A rectangular set of entries G_g[i0 + ii][j0 + jj], ii < ni, jj < nj, written
@@ -262,6 +285,14 @@ struct Operator {
     std::vector<int> sub_of_cluster_ptr, sub_of_cluster;   // per cluster: its sub-clusters
     std::vector<int> sub_start, sub_size, sub_tet_ptr;     // per sub-cluster
     int* d_sub_tets = nullptr;
+    double min_diam = 1e300;                               // smallest tetrahedron diameter
+    // tables of the row and column evaluation (rt_rows.cuh); freed when the assembly ends
+    std::vector<int> sub_pass0;                            // first pass of every sub-cluster
+    void* d_subs = nullptr;                                // SubInfo [sub-clusters]
+    unsigned short* d_pass_ref = nullptr;
+    unsigned* d_pass_run = nullptr;
+    std::vector<void*> eval_tables;                        // their allocations
+    int64_t eval_bytes = 0;
     std::vector<int> h_vt_ptr, h_vt_idx;                   // host copy of the vertex -> tetrahedra CSR
     // tensor-core multi-right-hand-side apply (one operator group, F % 16 == 0)
     int tc_enabled = 0;
@@ -295,11 +326,14 @@ struct Operator {
 
 // ---- kernels / drivers implemented in the .cu files -----------------------
 int assemble_setup_constants(Operator& op, std::string& err);
+// 4- and 14-point tetrahedron rules, 3- and 7-point triangle rules (barycentric points, weights)
+void quadrature_rules(double (&tet_b)[72], double (&tet_w)[18], double (&tri_b)[30], double (&tri_w)[10]);
 void gauss_legendre_nodes(int n, std::vector<double>& t, std::vector<double>& w);
 int assemble_dense(Operator& op, cudaStream_t s, std::string& err);
 int assemble_source(Operator& op, cudaStream_t s, std::string& err);
 int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err);
 int prepare_row_eval(Operator& op, std::string& err);
+void eval_tables_free(Operator& op);
 int eval_entries(Operator& op, int group, int64_t count, const int32_t* rows, const int32_t* cols, double* out,
                  cudaStream_t s, std::string& err);
 int hmatvec_prepare(Operator& op, std::string& err);

@@ -1,0 +1,69 @@
+"""Row and column evaluation (rt_rows.cuh): every evaluator and chunk width against the oracle.
+
+With eta tiny every leaf pair is a dense block, so an apply shows the row evaluation alone: pass and
+sub-cluster edges (tetrahedra per pass 128 or 512, leaves up to 256 columns), group chunks (1, 4, 8,
+16, several) and the three evaluators (phase tables: walls normal to an axis; plain: oblique walls, a
+wall that makes the domain's box too long, node sums; general: two walls, grid).  With eta = 2 the
+pivot columns take part.
+
+Tolerances.  FP32 entries carry about ten roundings of 6e-8 and an optical depth within 1e-6 of its
+value (the bound of the special-function sines), so an apply to positive vectors is within 2e-6 of the
+dense FP64 matrix in the 2-norm; ACA at eps = 1e-4 adds its own 1e-4 bound.
+"""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(n, groups, wall, kind="sin"):
+    rng = np.random.default_rng(n + 10 * groups)
+    kappa = W.sinprod_kappa(0.6) if kind != "const" else W.Kappa(W.KAPPA_CONST, 1.3, 0.0)
+    p = W.cube_problem(n, kappa, W.midpoint_freqs(groups, albedo=0.3), R0=0.0)
+    xyz = p.xyz.copy()
+    inner = ((xyz > 1e-9) & (xyz < 1 - 1e-9)).all(axis=1)
+    xyz[inner] += rng.uniform(-0.1, 0.1, size=(int(inner.sum()), 3)) / (n - 1)
+    p.xyz = xyz
+    if wall:
+        p.wall = W.Wall(*wall)
+    if kind == "uneven":
+        p.freqs.c = np.linspace(0.5, 1.0, groups) ** 2 + 0.3
+    if kind == "grid":
+        p.kappa = W.Kappa(W.KAPPA_GRID, 0.0, 0.0, rng.uniform(0.2, 2.0, size=(3, 4, 5)).astype(np.float32),
+                          (0.0, 0.0, 0.0, 1.0, 1.0, 1.0))
+        p.more_walls = (W.Wall((0.0, 0.0, 0.0), (0.0, -1.0, 0.0), 0.4),)
+        p.corner = True
+    return p
+
+
+Z0 = ((0.0, 0.0, 0.0), (0.0, 0.0, -1.0), 0.5)
+X1 = ((1.0, 0.3, 0.0), (2.0, 0.0, 0.0), 0.7)
+Y_OFF = ((0.0, -0.015, 0.0), (0.0, -1.0, 0.0), 0.6)
+OBLIQUE = ((0.0, 0.0, 0.0), (-0.3, -0.2, -1.0), 0.5)
+
+
+@pytest.mark.parametrize("n,groups,wall,kind,leaf", [
+    (2, 1, Z0, "sin", 64), (5, 1, None, "sin", 64), (8, 1, Z0, "sin", 256), (7, 1, X1, "const", 33),
+    (6, 2, X1, "sin", 64), (7, 4, Y_OFF, "sin", 31), (7, 5, Z0, "sin", 64), (6, 9, Z0, "uneven", 64),
+    (8, 16, Z0, "sin", 100), (6, 17, X1, "sin", 64), (5, 33, Z0, "sin", 64),
+    (6, 1, OBLIQUE, "sin", 64), (6, 8, OBLIQUE, "sin", 64), (6, 20, OBLIQUE, "sin", 64),
+    (6, 1, Z0, "grid", 64), (6, 6, Z0, "grid", 64), (5, 18, Z0, "grid", 64),
+])
+@pytest.mark.parametrize("eta", [1e-9, 2.0])
+def test_rows_and_columns_match_oracle(n, groups, wall, kind, leaf, eta):
+    import torch
+
+    import paper_2306_05789_gb300 as rt
+    from oracle import oracle as O
+    p = _problem(n, groups, wall, kind)
+    X = W.rand_vectors((groups, p.N), seed=1).astype(np.float32)
+    ref = O.DenseOperator(p).apply(X.astype(np.float64))
+    op = rt.rt_build_operator(p, rt.hparams(leaf=leaf, eta=eta))
+    Xd = torch.tensor(X, device="cuda")
+    Y = torch.empty_like(Xd)
+    op.apply(Xd, Y)
+    err = np.linalg.norm(Y.double().cpu().numpy() - ref) / np.linalg.norm(ref)
+    assert err < (2e-6 if eta < 1 else 1e-4)
+    op.free()
