@@ -526,11 +526,11 @@ int prepare_row_eval(Operator& op, std::string& err)
     return RT_EVALUATOR(op, tables(op, tets, err));
 }
 
-// most rows of one item: the sums of all its rows take at most 32 KB
-static int rows_per_item(int mg, int n) { return std::max(1, std::min(8, 32768 / (4 * mg * n))); }
+// rows of one item: the more, the wider the stores of a column's rows; the sums
+// of all its rows take at most 8 KB, which keeps four CTAs on an SM at 16 groups
+static int rows_per_item(int mg, int n) { return std::max(1, std::min(8, 8192 / (4 * mg * n))); }
 
-static int launch_rows(Operator& op, const std::vector<RowItem>& items, const int* istar, float* out, cudaStream_t s,
-                       std::string& err)
+static int launch_rows(Operator& op, const std::vector<RowItem>& items, float* out, cudaStream_t s, std::string& err)
 {
     if (items.empty()) return RT_OK;
     RowItem* d = nullptr;
@@ -540,7 +540,7 @@ static int launch_rows(Operator& op, const std::vector<RowItem>& items, const in
     for (const RowItem& it : items) sums = std::max(sums, it.nrow * op.sub_size[it.sub]);
     for (size_t k0 = 0; k0 < items.size(); k0 += (size_t)1 << 30) {
         const int n = (int)std::min<size_t>(items.size() - k0, (size_t)1 << 30);
-        const int rc = RT_EVALUATOR(op, rows(op, d + k0, n, sums, istar, out, s, err));
+        const int rc = RT_EVALUATOR(op, rows(op, d + k0, n, sums, out, s, err));
         if (rc) return rc;
     }
     RT_CUDA_TRY(cudaFreeAsync(d, s));
@@ -548,270 +548,9 @@ static int launch_rows(Operator& op, const std::vector<RowItem>& items, const in
 }
 
 // ---------------------------------------------------------------------------
-// Batched partially pivoted ACA (Section 2.1), pivots shared by all groups.
-//
-// Every admissible block b (m x n) is approximated for all groups g at once:
-//   step k: residual row  R_g = G_g[i*, :] - sum_{l<k} u_{g,l}[i*] v_{g,l}
-//           pivot column  j*  = argmax_j sum_g |R_g[j]| / w_g   (first index on ties)
-//           v_g = R_g / R_g[j*]           (skipped for a group whose pivot is 0)
-//           u_g = G_g[:, j*] - sum_{l<k} u_{g,l} v_{g,l}[j*]
-//           ||S_g||_F^2 += 2 sum_{l<k} (u_l.u)(v_l.v) + |u|^2 |v|^2      (FP64)
-//           group g done when |u_g| |v_g| <= eps ||S_g||_F
-//           next row i* = argmax over unused rows of sum_g |u_g[i]| / w_g
-// w_g = ||S_g||_F (1 before the first term) puts the groups on one scale.
-// A block stops when every group is done; when another term would make
-// r (m + n) >= m n, or the rank limit is reached, it is stored dense.
-// The first pivot row is the block's first row.
+// ACA of the admissible blocks (rt_aca.cuh) and the packing of its terms
 // ---------------------------------------------------------------------------
 namespace {
-
-enum { ACA_ACTIVE = 0, ACA_DONE = 1, ACA_DENSE = 2 };
-
-__device__ __forceinline__ unsigned long long score_key(float s, int idx)
-{
-    if (!(s >= 0.0f) || isinf(s)) s = 0.0f;
-    return ((unsigned long long)__float_as_uint(s) << 32) | (unsigned long long)(0xffffffffu - (unsigned)idx);
-}
-
-struct AcaDev {
-    int G;
-    int rmax;
-    double eps;
-    const FarBlock* blk;
-    int* istar;
-    int* jstar;
-    int* rank;
-    int* status;
-    double* norm2;      // [nfar][G]
-    float* wscale;      // [nfar][G]   score weights 1/w_g
-    float* inv;         // [nfar][G]
-    int64_t* uoff;      // [nfar][rmax]
-    int64_t* voff;      // [nfar][rmax]
-    unsigned char* used;   // [sum m]
-    int64_t* used_off;  // [nfar]
-    unsigned long long* key;   // [nfar]  row pivot key, then next-row key
-    unsigned* rowmax;   // [nfar][G]  max |R_g| of the current row (float bits)
-    double* dots;       // per step: [dot0 + l][G][2]  (u_l.u, v_l.v), l = rank -> (|u|^2, |v|^2)
-    float* pool;
-};
-
-__device__ __forceinline__ int find_active(const AcaActive* a, int na, int64_t e, int mode)
-{
-    int lo = 0, hi = na - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        const int64_t f = mode == 0 ? a[mid].first_row : a[mid].first_col;
-        if (f <= e) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// residual row: R_g[jj] -= sum_l u_{g,l}[i*] v_{g,l}[jj]; row key = argmax score.
-__global__ void aca_row_residual(AcaDev D, const AcaActive* act, int na, int64_t total, float* buf)
-{
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int ai = find_active(act, na, e, 0);
-        const AcaActive a = act[ai];
-        const int jj = (int)(e - a.first_row);
-        const int b = a.b, r = D.rank[b], is = D.istar[b];
-        // lanes of this warp on the same block combine their row maxima first:
-        // one atomic per block and group per warp instead of one per lane
-        const unsigned peers = __match_any_sync(__activemask(), b);
-        const bool leader = (threadIdx.x & 31) == __ffs(peers) - 1;
-        float score = 0.0f;
-        for (int g = 0; g < D.G; ++g) {
-            float v = buf[a.rbuf + (int64_t)g * a.n + jj];
-            for (int l = 0; l < r; ++l) {
-                const float* U = D.pool + D.uoff[(int64_t)b * D.rmax + l] + (int64_t)g * a.m;
-                const float* V = D.pool + D.voff[(int64_t)b * D.rmax + l] + (int64_t)g * a.n;
-                v -= U[is] * V[jj];
-            }
-            buf[a.rbuf + (int64_t)g * a.n + jj] = v;
-            score += fabsf(v) * D.wscale[(int64_t)b * D.G + g];
-            const unsigned mx = __reduce_max_sync(peers, isfinite(v) ? __float_as_uint(fabsf(v)) : 0u);
-            if (leader && mx) atomicMax(&D.rowmax[(int64_t)b * D.G + g], mx);
-        }
-        atomicMax(&D.key[b], score_key(score, jj));
-    }
-}
-
-// pivot column j*, 1/delta per group; a zero row is skipped.
-__global__ void aca_row_pivot(AcaDev D, AcaActive* act, int na, const float* buf)
-{
-    for (int ai = blockIdx.x * blockDim.x + threadIdx.x; ai < na; ai += gridDim.x * blockDim.x) {
-        AcaActive& a = act[ai];
-        const int b = a.b;
-        const unsigned long long k = D.key[b];
-        const float best = __uint_as_float((unsigned)(k >> 32));
-        const int j = (int)(0xffffffffu - (unsigned)(k & 0xffffffffu));
-        D.key[b] = 0ull;
-        if (!(best > 0.0f)) {
-            // exact zero row: mark it used and move to the next unused row
-            a.skip = 1;
-            D.used[D.used_off[b] + D.istar[b]] = 1;
-            int nxt = -1;
-            for (int i = 0; i < a.m; ++i)
-                if (!D.used[D.used_off[b] + i]) {
-                    nxt = i;
-                    break;
-                }
-            if (nxt < 0) D.status[b] = ACA_DONE;
-            else D.istar[b] = nxt;
-            continue;
-        }
-        a.skip = 0;
-        D.jstar[b] = j;
-        for (int g = 0; g < D.G; ++g) {
-            const float d = buf[a.rbuf + (int64_t)g * a.n + j];
-            const float rmx = __uint_as_float(D.rowmax[(int64_t)b * D.G + g]);
-            D.rowmax[(int64_t)b * D.G + g] = 0u;
-            // a group whose value at the shared pivot is negligible skips this term
-            D.inv[(int64_t)b * D.G + g] = (fabsf(d) > 1e-4f * rmx && fabsf(d) > 1e-37f) ? 1.0f / d : 0.0f;
-        }
-    }
-}
-
-// v_g = R_g * inv_g into the pool
-__global__ void aca_store_v(AcaDev D, const AcaActive* act, int na, int64_t total, const float* buf)
-{
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int ai = find_active(act, na, e, 0);
-        const AcaActive a = act[ai];
-        if (a.skip) continue;
-        const int jj = (int)(e - a.first_row);
-        for (int g = 0; g < D.G; ++g)
-            D.pool[a.voff + (int64_t)g * a.n + jj] =
-                buf[a.rbuf + (int64_t)g * a.n + jj] * D.inv[(int64_t)a.b * D.G + g];
-    }
-}
-
-// u_g = C_g - sum_l u_{g,l} v_{g,l}[j*]; next-row key over unused rows.
-__global__ void aca_col_residual(AcaDev D, const AcaActive* act, int na, int64_t total, const float* buf)
-{
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int ai = find_active(act, na, e, 1);
-        const AcaActive a = act[ai];
-        if (a.skip) continue;
-        const int ii = (int)(e - a.first_col);
-        const int b = a.b, r = D.rank[b], js = D.jstar[b];
-        float score = 0.0f;
-        for (int g = 0; g < D.G; ++g) {
-            float v = buf[a.cbuf + (int64_t)g * a.m + ii];
-            for (int l = 0; l < r; ++l) {
-                const float* U = D.pool + D.uoff[(int64_t)b * D.rmax + l] + (int64_t)g * a.m;
-                const float* V = D.pool + D.voff[(int64_t)b * D.rmax + l] + (int64_t)g * a.n;
-                v -= U[ii] * V[js];
-            }
-            if (D.inv[(int64_t)b * D.G + g] == 0.0f) v = 0.0f;
-            D.pool[a.uoff + (int64_t)g * a.m + ii] = v;
-            score += fabsf(v) * D.wscale[(int64_t)b * D.G + g];
-        }
-        if (ii != D.istar[b] && !D.used[D.used_off[b] + ii]) atomicMax(&D.key[b], score_key(score, ii));
-    }
-}
-
-// dots (u_l.u, v_l.v) for l = 0..rank (l = rank: the new term itself); one CTA per (block, l).
-struct DotItem {
-    int ai;
-    int l;
-};
-
-// one warp per (block, l).  The warp's lanes are split among the groups (gp
-// groups at a time, gp a power of two <= 4, so L = 32 / gp >= 8 lanes per
-// group and every load of a group still fills a whole 32-byte sector); each
-// group's two dot products then need a reduction over only L lanes: FP32
-// partial sums per lane (length / L terms), FP64 across lanes.
-__global__ void __launch_bounds__(256) aca_dots(AcaDev D, const AcaActive* act, const DotItem* items, int nitems)
-{
-    const int lane = threadIdx.x & 31;
-    int gp = 1;
-    while (gp < D.G && gp < 4) gp <<= 1;
-    const int L = 32 / gp;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t it = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitems; it += nw) {
-        const DotItem di = items[it];
-        const AcaActive a = act[di.ai];
-        if (a.skip) continue;
-        const int b = a.b;
-        const int64_t ul = di.l == D.rank[b] ? a.uoff : D.uoff[(int64_t)b * D.rmax + di.l];
-        const int64_t vl = di.l == D.rank[b] ? a.voff : D.voff[(int64_t)b * D.rmax + di.l];
-        for (int g0 = 0; g0 < D.G; g0 += gp) {
-            const int g = g0 + lane / L, sl = lane % L;
-            float pu = 0.f, pv = 0.f;
-            if (g < D.G) {
-                const float* U0 = D.pool + ul + (int64_t)g * a.m;
-                const float* U1 = D.pool + a.uoff + (int64_t)g * a.m;
-                const float* V0 = D.pool + vl + (int64_t)g * a.n;
-                const float* V1 = D.pool + a.voff + (int64_t)g * a.n;
-                // unrolled so that several loads per lane are in flight
-#pragma unroll 4
-                for (int i = sl; i < a.m; i += L) pu += U0[i] * U1[i];
-#pragma unroll 4
-                for (int j = sl; j < a.n; j += L) pv += V0[j] * V1[j];
-            }
-            double su = pu, sv = pv;
-            for (int o = L >> 1; o > 0; o >>= 1) {   // xor within aligned groups of L lanes
-                su += __shfl_xor_sync(0xffffffffu, su, o);
-                sv += __shfl_xor_sync(0xffffffffu, sv, o);
-            }
-            if (sl == 0 && g < D.G) {
-                double* dst = D.dots + ((a.dot0 + di.l) * D.G + g) * 2;
-                dst[0] = su;
-                dst[1] = sv;
-            }
-        }
-    }
-}
-
-__global__ void aca_finish(AcaDev D, const AcaActive* act, int na)
-{
-    for (int ai = blockIdx.x * blockDim.x + threadIdx.x; ai < na; ai += gridDim.x * blockDim.x) {
-        const AcaActive a = act[ai];
-        if (a.skip) continue;
-        const int b = a.b, r = D.rank[b];
-        bool all_done = true;
-        for (int g = 0; g < D.G; ++g) {
-            const double* dk = D.dots + ((a.dot0 + r) * D.G + g) * 2;
-            const double uu = dk[0], vv = dk[1];
-            double s = D.norm2[(int64_t)b * D.G + g];
-            double cross = 0.0;
-            for (int l = 0; l < r; ++l) {
-                const double* dl = D.dots + ((a.dot0 + l) * D.G + g) * 2;
-                cross += dl[0] * dl[1];
-            }
-            s += 2.0 * cross + uu * vv;
-            if (s < 0.0) s = 0.0;
-            D.norm2[(int64_t)b * D.G + g] = s;
-            // a group that skipped this shared pivot (1/delta = 0) has learned nothing
-            // from the term and is not declared converged by it
-            const bool skipped = D.inv[(int64_t)b * D.G + g] == 0.0f;
-            const bool done = !skipped && sqrt(uu * vv) <= D.eps * sqrt(s);
-            all_done = all_done && done;
-            D.wscale[(int64_t)b * D.G + g] = s > 0.0 ? (float)(1.0 / sqrt(s)) : 1.0f;
-        }
-        D.uoff[(int64_t)b * D.rmax + r] = a.uoff;
-        D.voff[(int64_t)b * D.rmax + r] = a.voff;
-        D.used[D.used_off[b] + D.istar[b]] = 1;
-        const int nr = r + 1;
-        D.rank[b] = nr;
-        const unsigned long long k = D.key[b];
-        D.key[b] = 0ull;
-        const float best = __uint_as_float((unsigned)(k >> 32));
-        if (all_done) {
-            D.status[b] = ACA_DONE;
-        } else if ((int64_t)(nr + 1) * (a.m + a.n) >= (int64_t)a.m * a.n || nr >= D.rmax) {
-            D.status[b] = ACA_DENSE;
-        } else if (k == 0ull || !(best > 0.0f)) {
-            // no unused row with a nonzero residual: the approximation is exact on all rows seen
-            D.status[b] = ACA_DONE;
-        } else {
-            D.istar[b] = (int)(0xffffffffu - (unsigned)(k & 0xffffffffu));
-        }
-    }
-}
 
 // repack converged blocks into V^T [G][r][n] and U^T [G][r][m] in the final storage type
 template <class T>
@@ -849,13 +588,13 @@ __global__ void aca_pack(AcaDev D, const PackItem* items, int nitems, const Chun
     __shared__ float red[2][32];
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const PackItem p = items[it];
-        const int64_t us = D.uoff[(int64_t)p.b * D.rmax + p.l], vs = D.voff[(int64_t)p.b * D.rmax + p.l];
+        const int64_t us = D.toff[(int64_t)p.b * D.rmax + p.l], vs = us + (int64_t)D.G * round4(p.m);
         for (int g = 0; g < D.G; ++g) {
             float su = 1.f;
             if (sizeof(T) == 2) {
                 float mu = 0.f, mv = 0.f;
-                for (int i = threadIdx.x; i < p.m; i += blockDim.x) mu = fmaxf(mu, fabsf(D.pool[us + (int64_t)g * p.m + i]));
-                for (int j = threadIdx.x; j < p.n; j += blockDim.x) mv = fmaxf(mv, fabsf(D.pool[vs + (int64_t)g * p.n + j]));
+                for (int i = threadIdx.x; i < p.m; i += blockDim.x) mu = fmaxf(mu, fabsf(D.pool[us + (int64_t)g * round4(p.m) + i]));
+                for (int j = threadIdx.x; j < p.n; j += blockDim.x) mv = fmaxf(mv, fabsf(D.pool[vs + (int64_t)g * round4(p.n) + j]));
                 for (int o = 16; o > 0; o >>= 1) {
                     mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, o));
                     mv = fmaxf(mv, __shfl_xor_sync(0xffffffffu, mv, o));
@@ -877,12 +616,12 @@ __global__ void aca_pack(AcaDev D, const PackItem* items, int nitems, const Chun
             const float sv = 1.f / su;
             for (int j = threadIdx.x; j < p.n; j += blockDim.x)
                 store_split<T>(dst, lo, p.voff_dst + ((int64_t)g * p.r + p.l) * p.n8 + j,
-                               sv * D.pool[vs + (int64_t)g * p.n + j]);
+                               sv * D.pool[vs + (int64_t)g * round4(p.n) + j]);
             for (int c = p.c0; c < p.c1; ++c) {
                 const Chunk ch = chunks[c];
                 for (int i = threadIdx.x; i < ch.m; i += blockDim.x)
                     store_split<T>(dst, lo, p.uoff_dst + ch.off + ((int64_t)g * p.r + p.l) * ch.m8 + i,
-                                   su * D.pool[us + (int64_t)g * p.m + ch.rbeg + i]);
+                                   su * D.pool[us + (int64_t)g * round4(p.m) + ch.rbeg + i]);
             }
         }
     }
@@ -926,7 +665,7 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
         tmp.clear();
     };
     float* pool = nullptr;
-    int64_t pool_cap = 0, pool_used = 0;
+    int64_t pool_cap = 0;
     float ms = 0.f, ms_pack = 0.f;
     const int esz = op.far_prec == RT_PREC_F32 ? 4 : 2;
     const bool split = op.refine && op.far_prec != RT_PREC_F32;
@@ -953,16 +692,14 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
     const int nwaves = (int)wave_start.size() - 1;
     op.info.aca_waves = nfar > 0 ? nwaves : 0;
     int nw_max = 0;
-    int64_t summ_max = 0, sumn_max = 0;
+    int64_t summ_max = 0;
     for (int w = 0; w < nwaves; ++w) {
-        int64_t sm = 0, sn = 0;
+        int64_t sm = 0;
         for (int b = wave_start[w]; b < wave_start[w + 1]; ++b) {
             sm += farb[b].m;
-            sn += farb[b].n;
         }
         nw_max = std::max(nw_max, wave_start[w + 1] - wave_start[w]);
         summ_max = std::max(summ_max, sm);
-        sumn_max = std::max(sumn_max, sn);
     }
 
     // final far storage layout, filled wave by wave
@@ -1005,32 +742,34 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
         FarBlock* d_blk;
         TA(d_blk, sizeof(FarBlock) * nw_max);
         TA(D.istar, sizeof(int) * nw_max);
-        TA(D.jstar, sizeof(int) * nw_max);
         TA(D.rank, sizeof(int) * nw_max);
+        TA(D.steps, sizeof(int) * nw_max);
         TA(D.status, sizeof(int) * nw_max);
         TA(D.norm2, sizeof(double) * nw_max * G);
         TA(D.wscale, sizeof(float) * nw_max * G);
-        TA(D.inv, sizeof(float) * nw_max * G);
-        TA(D.uoff, sizeof(int64_t) * nw_max * rmax);
-        TA(D.voff, sizeof(int64_t) * nw_max * rmax);
+        TA(D.toff, sizeof(int64_t) * nw_max * rmax);
         TA(D.used, summ_max);
         TA(D.used_off, sizeof(int64_t) * nw_max);
-        TA(D.key, sizeof(unsigned long long) * nw_max);
-        TA(D.rowmax, sizeof(unsigned) * nw_max * G);
+        int *d_order, *d_sub_ptr, *d_sub_of, *d_ctl;
+        TA(d_order, sizeof(int) * nw_max);
+        TA(d_sub_ptr, sizeof(int) * op.sub_of_cluster_ptr.size());
+        TA(d_sub_of, sizeof(int) * op.sub_of_cluster.size());
+        TA(d_ctl, 4 * sizeof(int));   // terms taken from the pool (8 bytes), next block, most steps
         D.blk = d_blk;
-        float *rowbuf, *colbuf;
-        TA(rowbuf, sizeof(float) * (size_t)G * sumn_max);
-        TA(colbuf, sizeof(float) * (size_t)G * summ_max);
-        AcaActive* d_act;
-        TA(d_act, sizeof(AcaActive) * nw_max);
-        DotItem* d_dot = nullptr;
-        double* d_dotv = nullptr;
-        int64_t dot_cap = 0;
+        D.order = d_order;
+        D.sub_ptr = d_sub_ptr;
+        D.sub_of = d_sub_of;
+        D.pool_used = (unsigned long long*)d_ctl;
+        D.next = d_ctl + 2;
+        D.max_steps = d_ctl + 3;
+        RT_CUDA_TRY(cudaMemcpyAsync(d_sub_ptr, op.sub_of_cluster_ptr.data(), sizeof(int) * op.sub_of_cluster_ptr.size(),
+                                    cudaMemcpyHostToDevice, s));
+        RT_CUDA_TRY(cudaMemcpyAsync(d_sub_of, op.sub_of_cluster.data(), sizeof(int) * op.sub_of_cluster.size(),
+                                    cudaMemcpyHostToDevice, s));
+        int widest = 1;
+        for (int c : op.sub_size) widest = std::max(widest, c);
         std::vector<int> h_status_buf((size_t)nw_max * 2);
         int* h_status = h_status_buf.data();
-        int dev = 0, sms = 148;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const std::vector<float> ones((size_t)nw_max * G, 1.0f);
         cudaEvent_t pk0, pk1;
         cudaEventCreate(&pk0);
@@ -1048,19 +787,17 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
             RT_CUDA_TRY(cudaMemcpyAsync(d_blk, fw, sizeof(FarBlock) * nb, cudaMemcpyHostToDevice, s));
             RT_CUDA_TRY(cudaMemsetAsync(D.istar, 0, sizeof(int) * nb, s));
             RT_CUDA_TRY(cudaMemsetAsync(D.rank, 0, sizeof(int) * nb, s));
+            RT_CUDA_TRY(cudaMemsetAsync(D.steps, 0, sizeof(int) * nb, s));
             RT_CUDA_TRY(cudaMemsetAsync(D.status, 0, sizeof(int) * nb, s));
             RT_CUDA_TRY(cudaMemsetAsync(D.norm2, 0, sizeof(double) * nb * G, s));
             RT_CUDA_TRY(cudaMemcpyAsync(D.wscale, ones.data(), sizeof(float) * nb * G, cudaMemcpyHostToDevice, s));
             RT_CUDA_TRY(cudaMemsetAsync(D.used, 0, sum_m, s));
             RT_CUDA_TRY(cudaMemcpyAsync(D.used_off, used_off.data(), sizeof(int64_t) * nb, cudaMemcpyHostToDevice, s));
-            RT_CUDA_TRY(cudaMemsetAsync(D.key, 0, sizeof(unsigned long long) * nb, s));
-            RT_CUDA_TRY(cudaMemsetAsync(D.rowmax, 0, sizeof(unsigned) * nb * G, s));
             std::vector<int> h_rank(nb, 0), status(nb, ACA_ACTIVE);
 
             // term pool of this wave: kWaveRank terms per block, grown if needed
-            pool_used = 0;
             pool_cap = 0;
-            for (int b = 0; b < nb; ++b) pool_cap += (int64_t)G * (fw[b].m + fw[b].n) * (int64_t)kWaveRank;
+            for (int b = 0; b < nb; ++b) pool_cap += aca_term_size(G, fw[b].m, fw[b].n) * (int64_t)kWaveRank;
             if (cudaMallocAsync((void**)&pool, sizeof(float) * pool_cap, s) != cudaSuccess) {
                 cleanup();
                 err = "cudaMalloc (ACA pool) failed";
@@ -1070,125 +807,63 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
             scratch += (int64_t)sizeof(float) * pool_cap;
             note_peak(0);
 
-            std::vector<AcaActive> act;
-            std::vector<DotItem> dots;
-            for (int step = 0; step < rmax + 64; ++step) {
-                act.clear();
-                int64_t fr = 0, fc = 0, bufr = 0, bufc = 0, need = 0;
-                for (int b = 0; b < nb; ++b)
-                    if (status[b] == ACA_ACTIVE) need += (int64_t)G * (fw[b].m + fw[b].n);
-                if (need == 0) break;
-                if (pool_used + need > pool_cap) {
-                    const int64_t ncap = std::max<int64_t>(pool_cap + pool_cap / 2, pool_used + need * 8);
-                    float* np = nullptr;
-                    if (cudaMallocAsync((void**)&np, sizeof(float) * ncap, s) != cudaSuccess) {
-                        cudaFreeAsync(pool, s);
-                        cleanup();
-                        err = "cudaMalloc (ACA pool growth) failed";
-                        return RT_ENOMEM;
-                    }
-                    RT_CUDA_TRY(cudaMemcpyAsync(np, pool, sizeof(float) * pool_used, cudaMemcpyDeviceToDevice, s));
-                    note_peak((int64_t)sizeof(float) * ncap);   // old and new pool both live here
-                    scratch += (int64_t)sizeof(float) * (ncap - pool_cap);
+            // largest blocks first, so that none starts late (counting sort by m + n)
+            {
+                int most = 0;
+                for (int b = 0; b < nb; ++b) most = std::max(most, fw[b].m + fw[b].n);
+                std::vector<int> first(most + 2, 0), order(nb);
+                for (int b = 0; b < nb; ++b) first[most - (fw[b].m + fw[b].n) + 1]++;
+                for (int k = 0; k <= most; ++k) first[k + 1] += first[k];
+                for (int b = 0; b < nb; ++b) order[first[most - (fw[b].m + fw[b].n)]++] = b;
+                RT_CUDA_TRY(cudaMemcpyAsync(d_order, order.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, s));
+            }
+            RT_CUDA_TRY(cudaMemsetAsync(d_ctl, 0, 4 * sizeof(int), s));
+            D.nb = nb;
+            for (bool more = true; more;) {
+                D.pool_cap = pool_cap;
+                RT_CUDA_TRY(cudaMemsetAsync(D.next, 0, sizeof(int), s));
+                if ((rc = RT_EVALUATOR(op, aca(op, D, widest, s, err)))) {
                     cudaFreeAsync(pool, s);
-                    pool = np;
-                    pool_cap = ncap;
-                    D.pool = pool;
+                    cleanup();
+                    return rc;
                 }
-                int64_t ndot = 0, nchunk = 0;
-                for (int b = 0; b < nb; ++b) {
-                    if (status[b] != ACA_ACTIVE) continue;
-                    AcaActive a{};
-                    a.b = b;
-                    a.row0 = fw[b].row0;
-                    a.m = fw[b].m;
-                    a.col0 = fw[b].col0;
-                    a.n = fw[b].n;
-                    a.first_row = fr;
-                    a.first_col = fc;
-                    a.rbuf = bufr;
-                    a.cbuf = bufc;
-                    a.uoff = pool_used;
-                    pool_used += (int64_t)G * a.m;
-                    a.voff = pool_used;
-                    pool_used += (int64_t)G * a.n;
-                    a.dot0 = ndot;
-                    ndot += h_rank[b] + 1;
-                    a.first_chunk = nchunk;
-                    nchunk += col_chunks(a.m);
-                    fr += a.n;
-                    fc += a.m;
-                    bufr += (int64_t)G * a.n;
-                    bufc += (int64_t)G * a.m;
-                    act.push_back(a);
-                }
-                const int na = (int)act.size();
-                RT_CUDA_TRY(cudaMemcpyAsync(d_act, act.data(), sizeof(AcaActive) * na, cudaMemcpyHostToDevice, s));
-                // 1. pivot rows: one CTA per (block, sub-cluster of its columns)
-                {
-                    std::vector<RowItem> ritems;
-                    for (const AcaActive& a : act) {
-                        const FarBlock& fb = fw[a.b];
-                        for (int e = op.sub_of_cluster_ptr[fb.sc]; e < op.sub_of_cluster_ptr[fb.sc + 1]; ++e) {
-                            const int sb = op.sub_of_cluster[e];
-                            RowItem it{};
-                            it.b = a.b;
-                            it.i = fb.row0;
-                            it.nrow = 1;
-                            it.sub = sb;
-                            it.out = a.rbuf + (op.sub_start[sb] - fb.col0);
-                            it.gs = fb.n;
-                            it.js = 1;
-                            ritems.push_back(it);
-                        }
-                    }
-                    if ((rc = launch_rows(op, ritems, D.istar, rowbuf, s, err))) {
-                        cleanup();
-                        return rc;
-                    }
-                }
-                const int eg_r = (int)std::min<int64_t>((fr + 255) / 256, (int64_t)sms * 32);
-                aca_row_residual<<<std::max(1, eg_r), 256, 0, s>>>(D, d_act, na, fr, rowbuf);
-                aca_row_pivot<<<(na + 127) / 128, 128, 0, s>>>(D, d_act, na, rowbuf);
-                aca_store_v<<<std::max(1, eg_r), 256, 0, s>>>(D, d_act, na, fr, rowbuf);
-                // 2. pivot columns: one CTA per 64-row chunk, the column's quadrature
-                // points tabulated once per chunk
-                {
-                    if ((rc = RT_EVALUATOR(op, columns(op, d_act, na, nchunk, D.jstar, colbuf, s, err)))) {
-                        cleanup();
-                        return rc;
-                    }
-                }
-                const int eg_c = (int)std::min<int64_t>((fc + 255) / 256, (int64_t)sms * 32);
-                aca_col_residual<<<std::max(1, eg_c), 256, 0, s>>>(D, d_act, na, fc, colbuf);
-                // 3. dots with all previous terms and the new one (per-step scratch)
-                dots.clear();
-                for (int ai = 0; ai < na; ++ai)
-                    for (int l = 0; l <= h_rank[act[ai].b]; ++l) dots.push_back({ai, l});
-                if ((int64_t)dots.size() > dot_cap) {
-                    if (d_dot) cudaFreeAsync(d_dot, s);
-                    if (d_dotv) cudaFreeAsync(d_dotv, s);
-                    scratch -= (int64_t)(sizeof(DotItem) + 2 * G * sizeof(double)) * dot_cap;
-                    dot_cap = (int64_t)dots.size() * 2;
-                    RT_CUDA_TRY(cudaMallocAsync((void**)&d_dot, sizeof(DotItem) * dot_cap, s));
-                    RT_CUDA_TRY(cudaMallocAsync((void**)&d_dotv, sizeof(double) * 2 * G * dot_cap, s));
-                    scratch += (int64_t)(sizeof(DotItem) + 2 * G * sizeof(double)) * dot_cap;
-                    note_peak(0);
-                }
-                D.dots = d_dotv;
-                RT_CUDA_TRY(cudaMemcpyAsync(d_dot, dots.data(), sizeof(DotItem) * dots.size(), cudaMemcpyHostToDevice, s));
-                aca_dots<<<(int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)dots.size() + 7) / 8, (int64_t)sms * 32)),
-                           256, 0, s>>>(D, d_act, d_dot, (int)dots.size());
-                aca_finish<<<(na + 127) / 128, 128, 0, s>>>(D, d_act, na);
-                RT_CUDA_TRY(cudaGetLastError());
+                int ctl[4];
                 RT_CUDA_TRY(cudaMemcpyAsync(h_status, D.status, sizeof(int) * nb, cudaMemcpyDeviceToHost, s));
                 RT_CUDA_TRY(cudaMemcpyAsync(h_status + nb, D.rank, sizeof(int) * nb, cudaMemcpyDeviceToHost, s));
+                RT_CUDA_TRY(cudaMemcpyAsync(ctl, d_ctl, sizeof(ctl), cudaMemcpyDeviceToHost, s));
                 RT_CUDA_TRY(cudaStreamSynchronize(s));
+                more = false;
+                int64_t need = 0;   // one more term for every block that is still active
                 for (int b = 0; b < nb; ++b) {
                     status[b] = h_status[b];
                     h_rank[b] = h_status[nb + b];
+                    if (status[b] == ACA_ACTIVE) {
+                        more = true;
+                        need += aca_term_size(G, fw[b].m, fw[b].n);
+                    }
                 }
-                ++aca_steps;
+                if (!more) {
+                    aca_steps += ctl[3];
+                    break;
+                }
+                // the pool ran out: a larger one, and the active blocks go on
+                const int64_t ncap = std::max<int64_t>(pool_cap + pool_cap / 2, pool_cap + need * 8);
+                float* np = nullptr;
+                if (cudaMallocAsync((void**)&np, sizeof(float) * ncap, s) != cudaSuccess) {
+                    cudaFreeAsync(pool, s);
+                    cleanup();
+                    err = "cudaMalloc (ACA pool growth) failed";
+                    return RT_ENOMEM;
+                }
+                RT_CUDA_TRY(cudaMemcpyAsync(np, pool, sizeof(float) * pool_cap, cudaMemcpyDeviceToDevice, s));
+                note_peak((int64_t)sizeof(float) * ncap);   // old and new pool both live here
+                scratch += (int64_t)sizeof(float) * (ncap - pool_cap);
+                cudaFreeAsync(pool, s);
+                const unsigned long long taken = (unsigned long long)pool_cap;
+                RT_CUDA_TRY(cudaMemcpyAsync(D.pool_used, &taken, sizeof(taken), cudaMemcpyHostToDevice, s));
+                pool = np;
+                pool_cap = ncap;
+                D.pool = pool;
             }
             // ---- this wave's blocks: stored low rank, all-zero, or dense ------
             const int64_t elems0 = far_elems;
@@ -1281,9 +956,6 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
             scratch -= (int64_t)sizeof(float) * pool_cap;
             pool = nullptr;
         }
-        if (d_dot) cudaFreeAsync(d_dot, s);
-        if (d_dotv) cudaFreeAsync(d_dotv, s);
-        scratch -= (int64_t)(sizeof(DotItem) + 2 * G * sizeof(double)) * dot_cap;
         cudaEventDestroy(pk0);
         cudaEventDestroy(pk1);
 #undef TA
@@ -1324,7 +996,6 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                     const int rows = rows_per_item(group_chunk(op), op.sub_size[sb]);
                     for (int ii = 0; ii < ch.m; ii += rows) {
                         RowItem it{};
-                        it.b = -1;
                         it.i = fb.row0 + ch.rbeg + ii;
                         it.nrow = std::min(rows, ch.m - ii);
                         it.sub = sb;
@@ -1336,7 +1007,7 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                 }
             }
         }
-        if ((rc = launch_rows(op, ritems, nullptr, op.d_near, s, err))) return rc;
+        if ((rc = launch_rows(op, ritems, op.d_near, s, err))) return rc;
         for (int k = 0; k < op.n_near; ++k)
             op.info.entries_evaluated += (int64_t)op.dense_blocks[k].m * op.dense_blocks[k].n;
     }

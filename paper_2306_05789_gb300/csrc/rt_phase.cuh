@@ -261,7 +261,7 @@ __device__ __forceinline__ void phase_direct(const KernelParams& P, const PhaseP
 #pragma unroll
             for (int m = 0; m < 4; ++m)
                 if (fabsf(d[m]) < kSmallDir) {
-                    n[m] = (float)(2.0 * kPi) * sin2pi(fmaf(0.5f, d[m], f[m])) * sinc_small(d[m]);
+                    n[m] = (float)(2.0 * kPi) * sin2pi_sfu(fmaf(0.5f, d[m], f[m])) * sinc_small(d[m]);
                     d[m] = 1.f;
                 }
         }
@@ -296,8 +296,8 @@ __device__ __forceinline__ void phase_reflected(const KernelParams& P, const Pha
             for (int m = 0; m < 4; ++m)
                 if (fabsf(d[m]) < kSmallRefl) {
                     const float a = t * d[m], b = s * d[m];
-                    n[m] = (float)(2.0 * kPi) * (t * sin2pi(fmaf(-0.5f, a, f[m])) * sinc_small(a) +
-                                                 s * sin2pi(fmaf(-0.5f, b, f[m ^ 1])) * sinc_small(b));
+                    n[m] = (float)(2.0 * kPi) * (t * sin2pi_sfu(fmaf(-0.5f, a, f[m])) * sinc_small(a) +
+                                                 s * sin2pi_sfu(fmaf(-0.5f, b, f[m ^ 1])) * sinc_small(b));
                     d[m] = 1.f;
                 }
         }

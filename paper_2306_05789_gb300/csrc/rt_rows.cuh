@@ -7,7 +7,7 @@
 // value at point q reaches vertex q with weight a and the others with b, so a
 // tetrahedron's four vertex sums are b S + (a - b) e_q with S = sum e_q: one
 // addition per point and group instead of four products.  The vertex sums go
-// to shared memory (kRowThreads tetrahedra a pass) and every column gathers
+// to shared memory (nth tetrahedra a pass) and every column gathers
 // its own from a list made once per operator: plain stores and loads in place
 // of 4 G shared float atomics per tetrahedron, which are compare-and-swap
 // loops that neighbouring tetrahedra contend for.
@@ -29,21 +29,47 @@
 
 namespace rt {
 
-constexpr int kRowThreads = 128;
+// add this thread's counts to the work counters (one atomic per warp and counter)
+__device__ __forceinline__ void count_work(const KernelParams& P, unsigned terms, unsigned depths)
+{
+    if (!P.work) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        terms += __shfl_xor_sync(0xffffffffu, terms, o);
+        depths += __shfl_xor_sync(0xffffffffu, depths, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(P.work, (unsigned long long)terms);
+        atomicAdd(P.work + 1, (unsigned long long)depths);
+    }
+}
+
+constexpr int nth = 128;
+// CTAs of the row and ACA kernels on an SM, by registers (16 groups: also by shared memory)
+constexpr int ctas_per_sm(int mg, int ev) { return ev != EV_PHASE ? (mg <= 16 ? 4 : 2) : (mg <= 4 ? 6 : (mg <= 8 ? 5 : 4)); }
+
 constexpr int kRunWords = kSubCols + 4;   // per pass: run count, runs, end mark
 
+// Threads of a row or ACA kernel's CTA are a launch parameter: 128, or more when
+// a problem has too few blocks to fill the chip (eval_threads in rt_rows.h).
+// max_threads is the most that the registers of an instance allow; 128-thread
+// CTAs then run six (1 and 4 groups), five (8) or four (16) to an SM.
+constexpr int max_threads(int mg, int ev) { return ev != EV_PHASE ? (mg <= 16 ? 512 : 256) : (mg <= 4 ? 768 : (mg <= 8 ? 640 : 512)); }
+
 // Shapes of one row pass: TPT tetrahedra per thread (one group: four, so that a
-// pass is worth its two barriers), PT per pass; stage row of a tetrahedron
-// padded so that its 16-byte stores fall into different banks.
+// pass is worth its two barriers), PT = TPT x threads per pass; stage row of a
+// tetrahedron padded so that its 16-byte stores fall into different banks.
 template <int MG, int EV>
 struct RowShape {
     static constexpr int TPT = MG == 1 && EV == EV_PHASE ? 4 : 1;
-    static constexpr int PT = kRowThreads * TPT;
     static constexpr int RS = MG == 1 ? 4 : 4 * MG + 4;
-    static constexpr int LIST = EV != EV_GENERAL && MG > 1 ? 1024 : 2048;
     static constexpr int TERMS = EV == EV_GENERAL ? 2 + kMaxXTerms : 2;   // most list entries per tetrahedron
-    static constexpr int kFixed = PT * RS * 4 + 4 * PT * 2 + kRunWords * 4 + LIST * 4;   // bytes besides the sums
-    static_assert(LIST > TERMS * PT, "one pass must fit the list");
+    static __host__ __device__ constexpr int list(int nt) { return 2 * TERMS * TPT * nt; }   // two passes
+    // shared bytes of nt threads besides the sums
+    static __host__ __device__ constexpr int fixed(int nt)
+    {
+        return TPT * nt * RS * 4 + 4 * TPT * nt * 2 + kRunWords * 4 + list(nt) * 4;
+    }
 };
 
 // Term t's value at y for a near pair or a general problem (original
@@ -114,11 +140,12 @@ struct RowShared {
     int* cnt;              // length of list
     __device__ RowShared(char* base, int* counter)
     {
+        const int nt = blockDim.x;
         stage = (float*)base;
-        ref = (uint16_t*)(stage + S::PT * S::RS);
-        run = (unsigned*)(ref + 4 * S::PT);
+        ref = (uint16_t*)(stage + S::TPT * nt * S::RS);
+        run = (unsigned*)(ref + 4 * S::TPT * nt);
         list = run + kRunWords;
-        acc = (float*)(list + S::LIST);
+        acc = (float*)(list + S::list(nt));
         cnt = counter;
     }
 };
@@ -130,7 +157,7 @@ __device__ __noinline__ void near_flush(const KernelParams& P, const SubInfo& su
 {
     using S = RowShape<MG, EV>;
     const int cnt = *sh.cnt;
-    for (int e = threadIdx.x; e < cnt; e += kRowThreads) {
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
         const unsigned ent = sh.list[e];
         const int r = ent >> 28, t = (ent >> 24) & 15, tet = sub_tets[sub.tet0 + (ent & 0xffffff)];
         const Vec3<float> xi = load_xyz<float>(P, i0 + r);
@@ -180,38 +207,38 @@ __device__ __forceinline__ void row_segment(const KernelParams& P, const SubInfo
                                             unsigned& n_depths)
 {
     using S = RowShape<MG, EV>;
-    const int tid = threadIdx.x;
-    for (int k = tid; k < nrow * sub.size * MG; k += kRowThreads) sh.acc[k] = 0.f;
+    constexpr int RW = (kRunWords + 127) / 128;
+    const int tid = threadIdx.x, nth = blockDim.x, PT = S::TPT * nth, list_cap = S::list(nth);
+    for (int k = tid; k < nrow * sub.size * MG; k += nth) sh.acc[k] = 0.f;
     if (tid == 0) *sh.cnt = 0;
     __syncthreads();
-    const int npass = (sub.ntet + S::PT - 1) / S::PT;
+    const int npass = (sub.ntet + PT - 1) / PT;
     for (int p = 0; p < npass; ++p) {
         // this pass's gather lists: fetched now, stored before the first barrier
         uint2 refs[S::TPT];
-        unsigned run_w[(kRunWords + kRowThreads - 1) / kRowThreads];
+        unsigned run_w[RW];
         {
-            const uint2* gr = reinterpret_cast<const uint2*>(pass_ref + (int64_t)(sub.pass0 + p) * 4 * S::PT);
+            const uint2* gr = reinterpret_cast<const uint2*>(pass_ref + (int64_t)(sub.pass0 + p) * 4 * PT);
             const unsigned* gw = pass_run + (int64_t)(sub.pass0 + p) * kRunWords;
 #pragma unroll
-            for (int k = 0; k < S::TPT; ++k) refs[k] = gr[k * kRowThreads + tid];
+            for (int k = 0; k < S::TPT; ++k) refs[k] = gr[k * nth + tid];
 #pragma unroll
-            for (int k = 0; k < (kRunWords + kRowThreads - 1) / kRowThreads; ++k)
-                run_w[k] = k * kRowThreads + tid < kRunWords ? gw[k * kRowThreads + tid] : 0u;
+            for (int k = 0; k < RW; ++k)
+                run_w[k] = k * nth + tid < kRunWords ? gw[k * nth + tid] : 0u;
         }
         for (int r = 0; r < nrow; ++r) {
             const int i = i0 + r;
             const Vec3<float> xi = load_xyz<float>(P, i);
 #pragma unroll 1
             for (int tt = 0; tt < S::TPT; ++tt) {
-                const int tl = p * S::PT + tt * kRowThreads + tid;
+                const int tl = p * PT + tt * nth + tid;
                 if (tl >= sub.ntet) break;
                 const int tet = sub_tets[sub.tet0 + tl];
                 const float4 cen4 = P.tcen[tet];
                 const Vec3<float> cen = {cen4.x, cen4.y, cen4.z};
-                float* row = sh.stage + (tt * kRowThreads + tid) * S::RS;
+                float* row = sh.stage + (tt * nth + tid) * S::RS;
                 GroupSum<MG> sum;
                 sum.zero();
-                float e1[4];   // one group: the point values stay in registers
                 if constexpr (EV == EV_PHASE) {
                     const PhasePoint x = phase_point(P, i);
                     const bool fd = !(dist2<float>(xi, cen) < cen4.w);
@@ -220,7 +247,7 @@ __device__ __forceinline__ void row_segment(const KernelParams& P, const SubInfo
                     if (P.has_wall && !fr) sh.list[atomicAdd(sh.cnt, 1)] = ((unsigned)r << 28) | (1u << 24) | (unsigned)tl;
                     n_terms += (fd ? 4 : 14) + (P.has_wall ? (fr ? 4 : 14) : 0);
                     n_depths += (fd ? 4 : 14) + (P.has_wall ? 2 * (fr ? 4 : 14) : 0);
-#pragma unroll(MG == 1 ? 4 : 1)
+#pragma unroll 1
                     for (int q = 0; q < 4; ++q) {
                         const float4 y4 = P.tpt[(int64_t)q * P.T + tet];
                         float4 yc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -237,8 +264,7 @@ __device__ __forceinline__ void row_segment(const KernelParams& P, const SubInfo
                             e.add(P, g0, w, tau);
                         }
                         sum.add(e);
-                        if constexpr (MG == 1) e1[q] = e.e;
-                        else e.store(row + q * MG);
+                        e.store(row + q * MG);
                     }
                 } else {
                     unsigned far = 0u;
@@ -255,7 +281,7 @@ __device__ __forceinline__ void row_segment(const KernelParams& P, const SubInfo
                         n_terms += nr ? 14 : 4;
                         n_depths += (nr ? 14 : 4) * legs;
                     }
-#pragma unroll(MG == 1 ? 4 : 1)
+#pragma unroll 1
                     for (int q = 0; q < 4; ++q) {
                         const float4 y4 = P.tpt[(int64_t)q * P.T + tet];
                         const Vec3<float> y = {y4.x, y4.y, y4.z};
@@ -270,14 +296,14 @@ __device__ __forceinline__ void row_segment(const KernelParams& P, const SubInfo
                             if (general_term<EV == EV_GENERAL>(P, t, xi, src, scale, y, y4.w, w, tau)) e.add(P, g0, w, tau);
                         }
                         sum.add(e);
-                        if constexpr (MG == 1) e1[q] = e.e;
-                        else e.store(row + q * MG);
+                        e.store(row + q * MG);
                     }
                 }
                 if constexpr (MG == 1) {
                     const float bs = kTetB * sum.e;
-                    *reinterpret_cast<float4*>(row) = make_float4(fmaf(kTetG, e1[0], bs), fmaf(kTetG, e1[1], bs),
-                                                                  fmaf(kTetG, e1[2], bs), fmaf(kTetG, e1[3], bs));
+                    float4 e = *reinterpret_cast<float4*>(row);
+                    e = make_float4(fmaf(kTetG, e.x, bs), fmaf(kTetG, e.y, bs), fmaf(kTetG, e.z, bs), fmaf(kTetG, e.w, bs));
+                    *reinterpret_cast<float4*>(row) = e;
                 } else {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) sum.blend(row + q * MG, kTetB, kTetG);
@@ -285,15 +311,15 @@ __device__ __forceinline__ void row_segment(const KernelParams& P, const SubInfo
             }
             if (r == 0) {
 #pragma unroll
-                for (int k = 0; k < S::TPT; ++k) reinterpret_cast<uint2*>(sh.ref)[k * kRowThreads + tid] = refs[k];
+                for (int k = 0; k < S::TPT; ++k) reinterpret_cast<uint2*>(sh.ref)[k * nth + tid] = refs[k];
 #pragma unroll
-                for (int k = 0; k < (kRunWords + kRowThreads - 1) / kRowThreads; ++k)
-                    if (k * kRowThreads + tid < kRunWords) sh.run[k * kRowThreads + tid] = run_w[k];
+                for (int k = 0; k < RW; ++k)
+                    if (k * nth + tid < kRunWords) sh.run[k * nth + tid] = run_w[k];
             }
             __syncthreads();
             // MG lanes per column run
             const int nrun = (int)sh.run[0], g = tid % MG;
-            for (int k = tid / MG; k < nrun; k += kRowThreads / MG) {
+            for (int k = tid / MG; k < nrun; k += nth / MG) {
                 const unsigned w0 = sh.run[1 + k];
                 const int a = w0 & 0xffff, b = sh.run[2 + k] & 0xffff;
                 float v = 0.f;
@@ -303,7 +329,7 @@ __device__ __forceinline__ void row_segment(const KernelParams& P, const SubInfo
             }
             const int cnt = *sh.cnt;
             __syncthreads();
-            if (cnt > S::LIST - S::TERMS * S::PT) near_flush<MG, EV>(P, sub, sub_tets, i0, g0, sh);
+            if (cnt > list_cap - S::TERMS * PT) near_flush<MG, EV>(P, sub, sub_tets, i0, g0, sh);
         }
     }
     near_flush<MG, EV>(P, sub, sub_tets, i0, g0, sh);
@@ -314,18 +340,18 @@ __device__ __forceinline__ void row_segment(const KernelParams& P, const SubInfo
 template <int MG, int EV>
 __global__ void __launch_bounds__(256) pass_lists_kernel(const int4* __restrict__ tet, const SubInfo* __restrict__ subs,
                                                          const int* __restrict__ pass_sub, const int* __restrict__ sub_tets,
-                                                         uint16_t* __restrict__ ref, unsigned* __restrict__ run)
+                                                         int PT, uint16_t* __restrict__ ref, unsigned* __restrict__ run)
 {
     using S = RowShape<MG, EV>;
-    __shared__ short loc[4 * S::PT];
+    extern __shared__ short loc[];   // [4 PT]
     __shared__ int scan[2][256];
     const SubInfo sub = subs[pass_sub[blockIdx.x]];
     const int p = blockIdx.x - sub.pass0, j = threadIdx.x;
-    const int nt = min(S::PT, sub.ntet - p * S::PT);
-    uint16_t* pref = ref + (int64_t)blockIdx.x * 4 * S::PT;
+    const int nt = min(PT, sub.ntet - p * PT);
+    uint16_t* pref = ref + (int64_t)blockIdx.x * 4 * PT;
     unsigned* prun = run + (int64_t)blockIdx.x * kRunWords;
     for (int t = j; t < nt; t += 256) {
-        const int4 tv = tet[sub_tets[sub.tet0 + p * S::PT + t]];
+        const int4 tv = tet[sub_tets[sub.tet0 + p * PT + t]];
         const int id[4] = {tv.x, tv.y, tv.z, tv.w};
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -355,8 +381,8 @@ __global__ void __launch_bounds__(256) pass_lists_kernel(const int4* __restrict_
 }
 
 // ---- pivot columns ---------------------------------------------------------------
-// Column j for rows row0 .. row0 + m - 1, up to 128 rows a call: with fewer than
-// 65 rows, several threads share a row's tetrahedra.  The column's points are
+// Column j for rows row0 .. row0 + m - 1, at most one row per thread a call: with
+// fewer rows, several threads share a row's tetrahedra.  The column's points are
 // the same for every row: a batch of kColTets tetrahedra is staged in shared
 // memory, and a warp's lanes read one point together.
 constexpr int kColTets = 32;
@@ -365,16 +391,17 @@ struct ColShared {
     float4 pt[kColTets][4], cs[kColTets][4];
     float4 cen[kColTets];
     int tet[kColTets];
-    float red[kColThreads * MG];
+    float red[1];   // [threads][MG], past the end of the struct
+    static constexpr int bytes(int nt) { return (int)sizeof(ColShared) + 4 * MG * nt; }
 };
 
-// out[g * gstride + row]: the finished sums times c_g, rows r0 .. r0 + mc - 1 (mc <= kColThreads)
+// out[g * gstride + row]: the finished sums times c_g, rows r0 .. r0 + mc - 1 (mc <= threads)
 template <int MG, int EV>
 __device__ __forceinline__ void column_chunk(const KernelParams& P, int row0, int mc, int j, int g0, ColShared<MG>& sh,
                                              float* __restrict__ out, int64_t gstride, unsigned& n_terms, unsigned& n_depths)
 {
-    const int tid = threadIdx.x;
-    const int parts = kColThreads / mc;
+    const int tid = threadIdx.x, nth = blockDim.x;
+    const int parts = nth / mc;
     const int part = tid / mc, pos = tid - part * mc;
     const bool live = part < parts;
     const int i = row0 + (live ? pos : 0);
@@ -385,7 +412,7 @@ __device__ __forceinline__ void column_chunk(const KernelParams& P, int row0, in
     for (int b0 = t0; b0 < t1; b0 += kColTets) {
         const int nt = min(kColTets, t1 - b0);
         __syncthreads();   // the previous batch is no longer read
-        for (int e = tid; e < nt * 4; e += kColThreads) {
+        for (int e = tid; e < nt * 4; e += nth) {
             const int t = e >> 2, q = e & 3;
             const int packed = P.vt_idx[b0 + t], tet = packed >> 2;
             float4 y4 = P.tpt[(int64_t)q * P.T + tet];
@@ -417,7 +444,7 @@ __device__ __forceinline__ void column_chunk(const KernelParams& P, int row0, in
                 if (P.has_wall && !fr) near[1] |= 1u << t;
                 n_terms += (fd ? 4 : 14) + (P.has_wall ? (fr ? 4 : 14) : 0);
                 n_depths += (fd ? 4 : 14) + (P.has_wall ? 2 * (fr ? 4 : 14) : 0);
-#pragma unroll(MG == 1 ? 2 : 1)
+#pragma unroll 1
                 for (int q = 0; q < 4; ++q) {
                     const float4 y4 = sh.pt[t][q], yc = sh.cs[t][q];
                     float w, tau;
@@ -484,7 +511,7 @@ __device__ __forceinline__ void column_chunk(const KernelParams& P, int row0, in
         __syncthreads();
         if (live) acc.store(sh.red + (part * mc + pos) * MG);
         __syncthreads();
-        for (int e = tid; e < mc * MG; e += kColThreads) {
+        for (int e = tid; e < mc * MG; e += nth) {
             const int g = e / mc, r = e - g * mc;
             if (g0 + g >= P.G) break;
             float v = 0.f;

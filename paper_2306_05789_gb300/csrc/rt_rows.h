@@ -8,23 +8,33 @@
 
 namespace rt {
 
-// ACA rows (mode 0) / columns (mode 1) of the active far blocks.
-struct AcaActive {
-    int b;          // far block id
-    int row0, m, col0, n;
-    int64_t rbuf;   // offset of this block's [G][n] row buffer
-    int64_t cbuf;   // offset of this block's [G][m] column buffer
-    int64_t first_row, first_col;   // prefix of n (rows) and m (cols) over the active list
-    int64_t uoff, voff;             // pool offsets of this step's u [G][m] and v [G][n]
-    int64_t dot0;                   // first entry of this block's rank+1 dot products this step
-    int64_t first_chunk;            // prefix of ceil(m / kColRows) over the active list
-    int skip;       // set by the pivot kernel: zero row, no rank this step
+// State of a wave of admissible blocks during ACA (rt_aca.cuh); block b of the
+// wave.  A term of block b: u [G][m4] then v [G][n4] at toff[b][l] of the pool,
+// rows padded with zeros to multiples of four for 16-byte loads.
+__host__ __device__ inline int round4(int x) { return (x + 3) & ~3; }
+inline int64_t aca_term_size(int G, int m, int n) { return (int64_t)G * (round4(m) + round4(n)); }
+enum { ACA_ACTIVE = 0, ACA_DONE = 1, ACA_DENSE = 2 };
+struct AcaDev {
+    int G, rmax, nb;
+    double eps;
+    const FarBlock* blk;
+    const int *sub_ptr, *sub_of;   // sub-clusters of every cluster
+    const int* order;   // [nb] largest blocks first
+    int* next;          // next entry of order to take
+    int* max_steps;
+    int *istar, *rank, *steps, *status;
+    double* norm2;      // [nb][G]
+    float* wscale;      // [nb][G]   score weights 1/w_g
+    int64_t* toff;      // [nb][rmax]
+    unsigned char* used;   // [sum m]
+    int64_t* used_off;  // [nb]
+    float* pool;
+    int64_t pool_cap;   // elements
+    unsigned long long* pool_used;
 };
-
 
 // Row segments: rows i .. i + nrow - 1 over one sub-cluster of columns.
 struct RowItem {
-    int b;            // ACA block (row = i + istar[b]) or -1 (rows i ...)
     int i, nrow;
     int sub;
     int64_t out;      // output offset of (first row, first column, group 0); rows are adjacent
@@ -36,10 +46,6 @@ struct SubInfo {
     int start, size, tet0, ntet, pass0;
 };
 
-// threads of a pivot-column CTA; the chunks of a block's rows are of equal size
-constexpr int kColThreads = 128;
-__host__ __device__ inline int col_chunks(int m) { return (m + kColThreads - 1) / kColThreads; }
-
 // Groups per chunk of the row and column kernels.  The phase evaluator's terms
 // cost about as much as 16 groups' exponentials and sums, and its chunks of 16
 // keep four CTAs on an SM; the others' terms cost several times that, so they
@@ -50,16 +56,26 @@ inline int group_chunk(const Operator& op)
     return G <= 1 ? 1 : (G <= 4 ? 4 : (G <= 8 ? 8 : (G <= 16 || op.kp.evaluator == EV_PHASE ? 16 : 32)));
 }
 
+// Threads of a row or ACA CTA.  One CTA runs a block's whole ACA, so with fewer
+// admissible blocks than the chip holds CTAs of 128 (about four on each of 152
+// SMs) more threads share a block: box with 298 blocks, ACA 417 ms with 128
+// threads, 150 ms with 512.
+inline int eval_threads(const Operator& op)
+{
+    const size_t nb = op.plan.far_blocks.size();
+    const int most = group_chunk(op) > 16 ? 256 : 512;
+    return nb >= 608 || nb == 0 ? 128 : (nb >= 304 ? 256 : most);
+}
+
 template <int EV>
 struct RowEval {
     // device tables (sub-clusters, gather lists, point tables) for the sub-clusters' tetrahedra
     static int tables(Operator& op, const std::vector<int>& tets, std::string& err);
     // rows of device items; sums: most (rows x columns) of one item
-    static int rows(Operator& op, const RowItem* items, int n, int sums, const int* istar, float* out, cudaStream_t s,
-                    std::string& err);
-    // pivot columns of the active blocks
-    static int columns(Operator& op, const AcaActive* act, int na, int64_t nchunks, const int* jstar, float* out,
-                       cudaStream_t s, std::string& err);
+    static int rows(Operator& op, const RowItem* items, int n, int sums, float* out, cudaStream_t s, std::string& err);
+    // ACA of the wave's active blocks, as far as the pool reaches; sums: columns of
+    // the widest sub-cluster
+    static int aca(Operator& op, const AcaDev& D, int sums, cudaStream_t s, std::string& err);
 };
 
 // CALL with EV the operator's evaluator

@@ -5,80 +5,29 @@
 #include <algorithm>
 #include <mutex>
 
-#include "rt_rows.cuh"
-#include "rt_rows.h"
+#include "rt_aca.cuh"
 
 namespace rt {
 
-// add this thread's counts to the work counters (one atomic per warp and counter)
-__device__ __forceinline__ void count_work(const KernelParams& P, unsigned terms, unsigned depths)
-{
-    if (!P.work) return;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        terms += __shfl_xor_sync(0xffffffffu, terms, o);
-        depths += __shfl_xor_sync(0xffffffffu, depths, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(P.work, (unsigned long long)terms);
-        atomicAdd(P.work + 1, (unsigned long long)depths);
-    }
-}
-
-// the active block holding row chunk e (first_chunk: prefix over the list)
-__device__ __forceinline__ int find_chunk(const AcaActive* a, int na, int64_t e)
-{
-    int lo = 0, hi = na - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (a[mid].first_chunk <= e) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// ACA pivot columns: G_g[i, j*] for the rows i of an active block, one CTA per
-// chunk of rows (blockIdx.y: chunk of MG groups).
 template <int MG, int EV>
-__global__ void __launch_bounds__(kColThreads) aca_col_kernel(KernelParams P, const AcaActive* __restrict__ act, int na,
-                                                              int64_t nchunks, const int* __restrict__ jstar,
-                                                              float* __restrict__ buf)
-{
-    __shared__ __align__(16) ColShared<MG> sh;
-    const int g0 = blockIdx.y * MG;
-    unsigned n_terms = 0, n_depths = 0;
-    for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-        const int ai = find_chunk(act, na, c);
-        const AcaActive a = act[ai];
-        if (a.skip) continue;   // CTA-uniform
-        const int nch = col_chunks(a.m), size = (a.m + nch - 1) / nch;
-        const int r0 = (int)(c - a.first_chunk) * size;
-        if (r0 >= a.m) continue;
-        column_chunk<MG, EV>(P, a.row0 + r0, min(size, a.m - r0), a.col0 + jstar[a.b], g0, sh, buf + a.cbuf + r0, a.m,
-                               n_terms, n_depths);
-    }
-    if (g0 == 0) count_work(P, n_terms, n_depths);
-}
-
-template <int MG, int EV>
-__global__ void __launch_bounds__(kRowThreads, MG <= 16 ? 4 : 2) row_items_kernel(KernelParams P, const RowItem* __restrict__ items,
+__global__ void __launch_bounds__(max_threads(MG, EV), 1) row_items_kernel(KernelParams P, const RowItem* __restrict__ items,
                                                                    const SubInfo* __restrict__ subs,
                                                                    const int* __restrict__ sub_tets,
                                                                    const uint16_t* __restrict__ pass_ref,
                                                                    const unsigned* __restrict__ pass_run,
-                                                                   const int* __restrict__ istar, float* __restrict__ out)
+                                                                   float* __restrict__ out)
 {
     extern __shared__ __align__(16) char smem[];
     __shared__ int cnt;
     const RowItem it = items[blockIdx.x];
     const SubInfo sub = subs[it.sub];
     const int g0 = blockIdx.y * MG, ng = min(MG, P.G - g0), n = sub.size;
-    const int i0 = it.b >= 0 ? it.i + istar[it.b] : it.i;
     const RowShared<MG, EV> sh(smem, &cnt);
     unsigned n_terms = 0, n_depths = 0;
-    row_segment<MG, EV>(P, sub, sub_tets, pass_ref, pass_run, i0, it.nrow, g0, sh, n_terms, n_depths);
+    row_segment<MG, EV>(P, sub, sub_tets, pass_ref, pass_run, it.i, it.nrow, g0, sh, n_terms, n_depths);
     if (g0 == 0) count_work(P, n_terms, n_depths);
     const int per = it.nrow * n;
-    for (int e = threadIdx.x; e < per * ng; e += kRowThreads) {
+    for (int e = threadIdx.x; e < per * ng; e += blockDim.x) {
         const int g = e / per, k = e - g * per;
         const int j = k / it.nrow, r = k - j * it.nrow;
         out[it.out + r + (int64_t)(g0 + g) * it.gs + (int64_t)j * it.js] = sh.acc[((int64_t)r * n + j) * MG + g] * P.cf[g0 + g];
@@ -114,7 +63,8 @@ int RowEval<EV>::tables(Operator& op, const std::vector<int>& tets, std::string&
     cudaStream_t s = op.stream;
     if ((rc = upload_rules(err))) return rc;
     int pt = 0;
-#define RT_PASS_TETS(MG, EV) pt = RowShape<MG, EV>::PT
+const int nth = eval_threads(op);
+#define RT_PASS_TETS(MG, EV) pt = RowShape<MG, EV>::TPT * nth
     RT_DISPATCH_MG(op, RT_PASS_TETS);
 #undef RT_PASS_TETS
     const int nsub = (int)op.sub_start.size();
@@ -156,7 +106,9 @@ int RowEval<EV>::tables(Operator& op, const std::vector<int>& tets, std::string&
     op.kp.tcos = cs;
     if (np > 0) {
 #define RT_PASS_LISTS(MG, EV) \
-    pass_lists_kernel<MG, EV><<<(unsigned)np, 256, 0, s>>>(op.d_tet, d_subs, d_pass_sub, op.d_sub_tets, op.d_pass_ref, op.d_pass_run)
+    pass_lists_kernel<MG, EV><<<(unsigned)np, 256, 4 * pt * sizeof(short), s>>>(op.d_tet, d_subs, d_pass_sub,       \
+                                                                                op.d_sub_tets, pt, op.d_pass_ref, \
+                                                                                op.d_pass_run)
         RT_DISPATCH_MG(op, RT_PASS_LISTS);
 #undef RT_PASS_LISTS
     }
@@ -168,12 +120,15 @@ int RowEval<EV>::tables(Operator& op, const std::vector<int>& tets, std::string&
     cudaGetDevice(&dev);
     if (dev < 64 && !attr_set[dev]) {
 #define RT_ROW_ATTR(MG, EV) \
-    RT_CUDA_TRY(cudaFuncSetAttribute(row_items_kernel<MG, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024))
+    RT_CUDA_TRY(cudaFuncSetAttribute(row_items_kernel<MG, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)); \
+    RT_CUDA_TRY(cudaFuncSetAttribute(aca_block_kernel<MG, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024))
         RT_ROW_ATTR(1, EV);
         RT_ROW_ATTR(4, EV);
         RT_ROW_ATTR(8, EV);
         RT_ROW_ATTR(16, EV);
-        if constexpr (EV != EV_PHASE) RT_ROW_ATTR(32, EV);
+        if constexpr (EV != EV_PHASE) {
+            RT_ROW_ATTR(32, EV);
+        }
 #undef RT_ROW_ATTR
         attr_set[dev] = true;
     }
@@ -181,15 +136,14 @@ int RowEval<EV>::tables(Operator& op, const std::vector<int>& tets, std::string&
 }
 
 template <int EV>
-int RowEval<EV>::rows(Operator& op, const RowItem* items, int n, int sums, const int* istar, float* out, cudaStream_t s,
-                      std::string& err)
+int RowEval<EV>::rows(Operator& op, const RowItem* items, int n, int sums, float* out, cudaStream_t s, std::string& err)
 {
-    const int mg = group_chunk(op);
+    const int mg = group_chunk(op), nth = eval_threads(op);
     const dim3 grid((unsigned)n, (op.G + mg - 1) / mg);
 #define RT_LAUNCH_ROWS(MG, EV)                                                                                  \
-    row_items_kernel<MG, EV><<<grid, kRowThreads, RowShape<MG, EV>::kFixed + (size_t)sums * MG * sizeof(float), \
+    row_items_kernel<MG, EV><<<grid, nth, RowShape<MG, EV>::fixed(nth) + (size_t)sums * MG * sizeof(float), \
                                s>>>(op.kp, items, (const SubInfo*)op.d_subs, op.d_sub_tets, op.d_pass_ref,      \
-                                    op.d_pass_run, istar, out)
+                                    op.d_pass_run, out)
     RT_DISPATCH_MG(op, RT_LAUNCH_ROWS);
 #undef RT_LAUNCH_ROWS
     RT_CUDA_TRY(cudaGetLastError());
@@ -197,14 +151,22 @@ int RowEval<EV>::rows(Operator& op, const RowItem* items, int n, int sums, const
 }
 
 template <int EV>
-int RowEval<EV>::columns(Operator& op, const AcaActive* act, int na, int64_t nchunks, const int* jstar, float* out,
-                         cudaStream_t s, std::string& err)
+int RowEval<EV>::aca(Operator& op, const AcaDev& D, int sums, cudaStream_t s, std::string& err)
 {
-    const int mg = group_chunk(op);
-    const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(nchunks, 152 * 32)), (op.G + mg - 1) / mg);
-#define RT_LAUNCH_COLUMNS(MG, EV) aca_col_kernel<MG, EV><<<grid, kColThreads, 0, s>>>(op.kp, act, na, nchunks, jstar, out)
-    RT_DISPATCH_MG(op, RT_LAUNCH_COLUMNS);
-#undef RT_LAUNCH_COLUMNS
+    const int nth = eval_threads(op);
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, op.device);
+#define RT_LAUNCH_ACA(MG, EV)                                                                                         \
+    do {                                                                                                              \
+        const size_t bytes = aca_phase_bytes<MG, EV>(nth) + (size_t)sums * MG * sizeof(float);                           \
+        int per_sm = 1;                                                                                               \
+        RT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, aca_block_kernel<MG, EV>, nth, bytes)); \
+        const int grid = std::max(1, std::min(D.nb, std::max(1, per_sm) * sms));                                      \
+        aca_block_kernel<MG, EV><<<grid, nth, bytes, s>>>(op.kp, D, (const SubInfo*)op.d_subs, op.d_sub_tets, \
+                                                                  op.d_pass_ref, op.d_pass_run);                      \
+    } while (0)
+    RT_DISPATCH_MG(op, RT_LAUNCH_ACA);
+#undef RT_LAUNCH_ACA
     RT_CUDA_TRY(cudaGetLastError());
     return RT_OK;
 }

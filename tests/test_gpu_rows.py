@@ -67,3 +67,27 @@ def test_rows_and_columns_match_oracle(n, groups, wall, kind, leaf, eta):
     err = np.linalg.norm(Y.double().cpu().numpy() - ref) / np.linalg.norm(ref)
     assert err < (2e-6 if eta < 1 else 1e-4)
     op.free()
+
+
+@pytest.mark.parametrize("groups", [1, 6])
+def test_aca_resumes_when_the_term_pool_runs_out(groups):
+    """eps = 1e-6 needs more terms than the pool first holds (24 a block): blocks stop, the pool grows,
+    they go on (one group: ranks above 24).  With six groups every block here ends dense."""
+    import torch
+
+    import paper_2306_05789_gb300 as rt
+    from oracle import oracle as O
+    p = _problem(11, groups, Z0)
+    X = W.rand_vectors((groups, p.N), seed=1).astype(np.float32)
+    rows = np.arange(0, p.N, 7, dtype=np.int32)
+    c, g = np.unique(np.asarray(p.freqs.c), return_inverse=True)
+    ref = np.stack([np.einsum("ij,j->i", np.asarray(O.G_rows(p, rows, c=c))[:, g[f]], X[f].astype(np.float64))
+                    for f in range(groups)])
+    for wave_bytes in (0, 1 << 20):
+        op = rt.rt_build_operator(p, rt.hparams(leaf=40, aca_eps=1e-6, wave_bytes=wave_bytes))
+        Xd = torch.tensor(X, device="cuda")
+        Y = torch.empty_like(Xd)
+        op.apply(Xd, Y)
+        got = Y.double().cpu().numpy()[:, rows]
+        assert np.linalg.norm(got - ref) < 4e-6 * np.linalg.norm(ref)
+        op.free()
