@@ -326,15 +326,46 @@ int hmatvec_prepare(Operator& op, std::string& err)
             err = "leaf clusters larger than 1024 rows are not supported";
             return RT_EINVAL;
         }
+    // algorithmic bytes of one apply: operator data once per frequency, X read, Y written
+    const int esz_far = op.far_prec == RT_PREC_F32 ? 4 : 2;
+    int64_t far_e = 0, near_e = 0;
+    for (int b = 0; b < op.n_far; ++b) far_e += (int64_t)op.rank[b] * (op.far_blocks[b].m + op.far_blocks[b].n);
+    for (int b = 0; b < op.n_near; ++b) near_e += (int64_t)op.dense_blocks[b].m * op.dense_blocks[b].n;
+    op.info.apply_bytes = F * (far_e * esz_far + near_e * 4) + 2 * F * N * (int64_t)esz;
+    op.info.apply_flops = 2 * F * (far_e + near_e);
+    if ((rc = tc_prepare(op, err))) return rc;
+    op.info.apply_tensor_cores = op.tc_enabled;
+    if (op.tc_enabled)   // one operator serves all F right-hand sides: its data is read once per apply
+        op.info.apply_bytes = far_e * esz_far + near_e * 4 + 2 * F * N * (int64_t)esz;
+    if ((rc = dev_alloc(op, &op.apply_err, 1, err))) return rc;
+    RT_CUDA_TRY(cudaMemsetAsync(op.apply_err, 0, sizeof(int), op.stream));
+    // the streamed tcgen05 apply serves every apply of its operators, refinement
+    // sweeps included (tc_serves): they need none of the CUDA-core work lists
+    // (41^3: 112 ms of host time)
+    if (op.tc2) return RT_OK;
     // ---- phase-1 rows and items ----------------------------------------------
+    // rows in order of falling length, a block's rows together: counting sort of the
+    // blocks (the rows themselves, sorted one by one, took 77 ms at 41^3)
+    std::vector<int> by_len(op.n_far);
+    {
+        int most = 0;
+        for (const FarBlock& fb : op.far_blocks) most = std::max(most, fb.n);
+        std::vector<int> first(most + 2, 0);
+        for (const FarBlock& fb : op.far_blocks) first[most - fb.n + 1]++;
+        for (int k = 0; k <= most; ++k) first[k + 1] += first[k];
+        for (int b = 0; b < op.n_far; ++b) by_len[first[most - op.far_blocks[b].n]++] = b;
+    }
     std::vector<P1Row> rows;
     std::vector<int64_t> w_base(op.n_far);
     int64_t wl = 0;
     for (int b = 0; b < op.n_far; ++b) {
+        w_base[b] = wl;
+        wl += F * op.rank[b];
+    }
+    rows.reserve((size_t)(wl / F));
+    for (int b : by_len) {
         const FarBlock& fb = op.far_blocks[b];
         const int r = op.rank[b];
-        w_base[b] = wl;
-        wl += F * r;
         for (int k = 0; k < r; ++k) {
             P1Row rw{};
             rw.v = op.far_v_off[b] + (int64_t)k * round8(fb.n);
@@ -346,10 +377,8 @@ int hmatvec_prepare(Operator& op, std::string& err)
             rows.push_back(rw);
         }
     }
-    std::stable_sort(rows.begin(), rows.end(), [](const P1Row& a, const P1Row& b) { return a.n > b.n; });
     std::vector<P1Item> items;
     const int vw = op.far_prec == RT_PREC_F32 ? 4 : 8;
-    const int esz_far = op.far_prec == RT_PREC_F32 ? 4 : 2;
     for (size_t i = 0; i < rows.size();) {
         const int n = rows[i].n;
         int sw = 32;
@@ -427,19 +456,7 @@ int hmatvec_prepare(Operator& op, std::string& err)
     op.n_p2_segs = (int)segs.size();
     op.w_len = wl;
     if ((rc = dev_alloc(op, &op.d_w, (size_t)std::max<int64_t>(wl, 1), err))) return rc;
-    if ((rc = dev_alloc(op, &op.apply_err, 1, err))) return rc;
-    RT_CUDA_TRY(cudaMemsetAsync(op.apply_err, 0, sizeof(int), op.stream));
     if ((rc = hs_prepare(op, w_base, per_leaf, leaves, esz_far, err))) return rc;
-    // algorithmic bytes of one apply: operator data once per frequency, X read, Y written
-    int64_t far_e = 0, near_e = 0;
-    for (int b = 0; b < op.n_far; ++b) far_e += (int64_t)op.rank[b] * (op.far_blocks[b].m + op.far_blocks[b].n);
-    for (int b = 0; b < op.n_near; ++b) near_e += (int64_t)op.dense_blocks[b].m * op.dense_blocks[b].n;
-    op.info.apply_bytes = F * (far_e * esz_far + near_e * 4) + 2 * F * N * (int64_t)esz;
-    op.info.apply_flops = 2 * F * (far_e + near_e);
-    if ((rc = tc_prepare(op, err))) return rc;
-    op.info.apply_tensor_cores = op.tc_enabled;
-    if (op.tc_enabled)   // one operator serves all F right-hand sides: its data is read once per apply
-        op.info.apply_bytes = far_e * esz_far + near_e * 4 + 2 * F * N * (int64_t)esz;
     return RT_OK;
 }
 
