@@ -128,36 +128,6 @@ int assemble_setup_constants(Operator& op, std::string& err)
 // ---------------------------------------------------------------------------
 constexpr int kWarpsPerCta = 8;
 
-__device__ __forceinline__ int find_span(const EntrySpan* sp, int ns, int64_t e)
-{
-    int lo = 0, hi = ns - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (sp[mid].first <= e) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-template <class R, class OUT, int MG, bool XT = false>
-__global__ void __launch_bounds__(32 * kWarpsPerCta) entries_span_kernel(KernelParams P, const EntrySpan* spans,
-                                                                         int nspans, int64_t total, OUT* out)
-{
-    __shared__ int s_tet[kWarpsPerCta][32], s_cnt[kWarpsPerCta][32], s_pre[kWarpsPerCta][33];
-    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * kWarpsPerCta;
-    for (int64_t e = (int64_t)blockIdx.x * kWarpsPerCta + wib; e < total; e += nw) {
-        const int si = find_span(spans, nspans, e);
-        const EntrySpan sp = spans[si];
-        const int64_t loc = e - sp.first;
-        const int ii = (int)(loc / sp.nj), jj = (int)(loc % sp.nj);
-        R acc[MG];
-        entry_warp<R, MG, XT>(P, sp.i0 + ii, sp.j0 + jj, acc, s_tet[wib], s_cnt[wib], s_pre[wib]);
-#pragma unroll
-        for (int g = 0; g < MG; ++g)
-            if (g < P.G && lane == (g & 31)) out[sp.base + g * sp.gs + ii * sp.is + jj * sp.js] = (OUT)acc[g];
-    }
-}
-
 // Arbitrary (row, col) pairs, internal vertex ids.
 template <class R, int MG, bool XT = false>
 __global__ void __launch_bounds__(32 * kWarpsPerCta) entries_pairs_kernel(KernelParams P, int group, int64_t count,
@@ -222,70 +192,154 @@ static int grid_for(int64_t warps)
         }                        \
     } while (0)
 
-template <class R, class OUT>
-static int launch_spans(Operator& op, const std::vector<EntrySpan>& spans_in, OUT* out, cudaStream_t s,
-                        std::string& err)
-{
-    if (spans_in.empty()) return RT_OK;
-    std::vector<EntrySpan> spans = spans_in;
-    int64_t total = 0;
-    for (auto& sp : spans) {
-        sp.first = total;
-        total += (int64_t)sp.ni * sp.nj;
-    }
-    EntrySpan* d_sp = nullptr;
-    RT_CUDA_TRY(cudaMallocAsync((void**)&d_sp, spans.size() * sizeof(EntrySpan), s));
-    RT_CUDA_TRY(cudaMemcpyAsync(d_sp, spans.data(), spans.size() * sizeof(EntrySpan), cudaMemcpyHostToDevice, s));
-    int grid = grid_for(total);
-    const int ns = (int)spans.size();
-#define RT_LAUNCH_SPANS(MG, XT) \
-    entries_span_kernel<R, OUT, MG, XT><<<grid, 32 * kWarpsPerCta, 0, s>>>(op.kp, d_sp, ns, total, out)
-#define RT_LAUNCH_SPANS1(MG) RT_LAUNCH_SPANS(MG, false)
-    if (op.kp.ext) RT_DISPATCH_MG_XT(op.G, RT_LAUNCH_SPANS);
-    else RT_DISPATCH_MG(op.G, RT_LAUNCH_SPANS1);
-#undef RT_LAUNCH_SPANS1
-#undef RT_LAUNCH_SPANS
-    RT_CUDA_TRY(cudaGetLastError());
-    RT_CUDA_TRY(cudaFreeAsync(d_sp, s));
-    op.info.entries_evaluated += total;
-    return RT_OK;
-}
-
 // ---------------------------------------------------------------------------
 // dense mode: the whole matrix [G][N][N] row-major
 // ---------------------------------------------------------------------------
+// A thread takes one tetrahedron of one row and evaluates every point once for
+// the four hat functions of its vertices (entry by entry, each point was
+// evaluated four times); the vertex sums go to scratch [row][vertex slot][g][T]
+// and dense_gather adds each column's in the order of its tetrahedra.
+// Bound: FP64 issue (1/64 of the FP32 rate): for a constant kappa a term is one
+// rsqrt (1/r^2 and r, and the broken path is as long as the line from the image)
+// and one exponential.  12^3, kappa = 1, one wall, 1.2e8 terms: the whole matrix
+// 117 ms entry by entry, 15.2 ms this way.
+template <class R>
+__device__ __forceinline__ R rsqrt_r(R x);
+template <>
+__device__ __forceinline__ float rsqrt_r<float>(float x) { return rsqrtf(x); }
+template <>
+__device__ __forceinline__ double rsqrt_r<double>(double x) { return rsqrt(x); }
+
+constexpr int kDenseThreads = 128;
+template <class R, int MG, bool XT>
+__global__ void __launch_bounds__(kDenseThreads) dense_tets_kernel(KernelParams P, int row0, int g0, R* __restrict__ scratch)
+{
+    const int tet = blockIdx.x * kDenseThreads + threadIdx.x;
+    if (tet >= P.T) return;
+    const Vec3<R> xi = load_xyz<R>(P, row0 + blockIdx.y);
+    Vec3<R> xb = xi;
+    if (P.has_wall) xb = mirror_point<R>(P, xi);
+    const int4 tv = P.tet[tet];
+    const Vec3<R> v[4] = {load_xyz<R>(P, tv.x), load_xyz<R>(P, tv.y), load_xyz<R>(P, tv.z), load_xyz<R>(P, tv.w)};
+    Vec3<R> cen;
+    R diam, vol;
+    load_tgeo<R>(P, tet, cen, diam, vol);
+    const R lim = R(4) * diam * diam, inv4pi = R(1.0 / (4.0 * kPi));
+    R acc[4][MG];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int g = 0; g < MG; ++g) acc[k][g] = R(0);
+    const int nt = XT ? 2 + P.n_extra : 2;
+    for (int t = 0; t < nt; ++t) {
+        if (t == 1 && !P.has_wall) continue;
+        Vec3<R> src;
+        R scale;
+        term_source<R>(P, t, xi, xb, src, scale);
+        const bool near = dist2<R>(src, cen) < lim;
+        const int q0 = near ? 4 : 0, nq = near ? 14 : 4;
+        for (int q = q0; q < q0 + nq; ++q) {
+            const R b[4] = {tet_b<R>(q, 0), tet_b<R>(q, 1), tet_b<R>(q, 2), tet_b<R>(q, 3)};
+            const Vec3<R> y = {b[0] * v[0].x + b[1] * v[1].x + b[2] * v[2].x + b[3] * v[3].x,
+                               b[0] * v[0].y + b[1] * v[1].y + b[2] * v[2].y + b[3] * v[3].y,
+                               b[0] * v[0].z + b[1] * v[1].z + b[2] * v[2].z + b[3] * v[3].z};
+            const R r2 = dist2<R>(src, y);
+            R w = scale * vol * tet_w<R>(q) * kappa_at<R, XT>(P, y.x, y.y, y.z) * inv4pi, tau;
+            if (!XT && P.kappa_kind == RT_KAPPA_CONST) {
+                const R rs = rsqrt_r<R>(r2);
+                tau = kp_k0<R>(P) * r2 * rs;
+                w *= rs * rs;
+            } else {
+                if constexpr (XT) {
+                    tau = term_depth<R>(P, t, xi, src, y);
+                    if (!(tau < R(INFINITY))) continue;   // path through an opaque box
+                } else if (t == 0) {
+                    tau = optical_depth<R>(P, xi, y);
+                } else {
+                    const Vec3<R> xp = wall_point<R>(P, src, y);
+                    tau = optical_depth<R>(P, xi, xp) + optical_depth<R>(P, xp, y);
+                }
+                w /= r2;
+            }
+#pragma unroll
+            for (int g = 0; g < MG; ++g)
+                if (g0 + g < P.G) {
+                    const R cg = kp_c<R>(P, g0 + g);
+                    const R e = w * cg * exp_r(-cg * tau);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[k][g] += b[k] * e;
+                }
+        }
+    }
+    const int64_t row = (int64_t)blockIdx.y * 4 * MG;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int g = 0; g < MG; ++g) scratch[(row + k * MG + g) * P.T + tet] = acc[k][g];
+}
+
+template <class R, int MG>
+__global__ void __launch_bounds__(256) dense_gather(KernelParams P, int row0, int g0, const R* __restrict__ scratch, R* __restrict__ out)
+{
+    const int j = blockIdx.x * 256 + threadIdx.x;
+    if (j >= P.N) return;
+    const int t0 = P.vt_ptr[j], t1 = P.vt_ptr[j + 1];
+    const int64_t row = (int64_t)blockIdx.y * 4 * MG;
+    for (int g = 0; g < MG && g0 + g < P.G; ++g) {
+        R s = R(0);
+#pragma unroll 4
+        for (int e = t0; e < t1; ++e) {
+            const int packed = P.vt_idx[e];
+            s += scratch[(row + (packed & 3) * MG + g) * P.T + (packed >> 2)];
+        }
+        out[(int64_t)(g0 + g) * P.N * P.N + (int64_t)(row0 + blockIdx.y) * P.N + j] = s;
+    }
+}
+
+template <class R, int MG>
+static int dense_rows(Operator& op, R* out, cudaStream_t s, std::string& err)
+{
+    // rows at a time: 64 MB of vertex sums stay in L2 between the two kernels
+    const int64_t per_row = (int64_t)4 * MG * op.T * sizeof(R);
+    const int rows = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(op.N, 32768), ((int64_t)64 << 20) / per_row));
+    R* scratch = nullptr;
+    if (cudaMallocAsync((void**)&scratch, (size_t)(rows * per_row), s) != cudaSuccess) {
+        err = "cudaMallocAsync (dense assembly scratch) failed";
+        return RT_ENOMEM;
+    }
+    for (int r0 = 0; r0 < op.N; r0 += rows) {
+        const int nr = std::min(rows, op.N - r0);
+        const dim3 ge((op.T + kDenseThreads - 1) / kDenseThreads, nr), gg((op.N + 255) / 256, nr);
+        for (int g0 = 0; g0 < op.G; g0 += MG) {
+            if (op.kp.ext) dense_tets_kernel<R, MG, true><<<ge, kDenseThreads, 0, s>>>(op.kp, r0, g0, scratch);
+            else dense_tets_kernel<R, MG, false><<<ge, kDenseThreads, 0, s>>>(op.kp, r0, g0, scratch);
+            dense_gather<R, MG><<<gg, 256, 0, s>>>(op.kp, r0, g0, scratch, out);
+        }
+    }
+    cudaFreeAsync(scratch, s);
+    RT_CUDA_TRY(cudaGetLastError());
+    return RT_OK;
+}
+
+template <class R>
+static int dense_matrix(Operator& op, cudaStream_t s, std::string& err)
+{
+    R* d = nullptr;
+    int rc = dev_alloc(op, &d, (size_t)op.G * op.N * op.N, err);
+    if (rc) return rc;
+    op.d_dense = d;
+    if (op.G <= 1) return dense_rows<R, 1>(op, d, s, err);
+    if (op.G <= 4) return dense_rows<R, 4>(op, d, s, err);
+    return dense_rows<R, 16>(op, d, s, err);
+}
+
 int assemble_dense(Operator& op, cudaStream_t s, std::string& err)
 {
     const int64_t N = op.N;
     const size_t esz = op.prec == RT_PREC_F64 ? 8 : 4;
-    int rc;
-    if (op.prec == RT_PREC_F64) {
-        double* d = nullptr;
-        if ((rc = dev_alloc(op, &d, (size_t)op.G * N * N, err))) return rc;
-        op.d_dense = d;
-    } else {
-        float* d = nullptr;
-        if ((rc = dev_alloc(op, &d, (size_t)op.G * N * N, err))) return rc;
-        op.d_dense = d;
-    }
-    // one span per row band keeps every span's entry count below 2^31
-    std::vector<EntrySpan> spans;
-    const int band = (int)std::max<int64_t>(1, std::min<int64_t>(N, (1 << 26) / std::max<int64_t>(N, 1)));
-    for (int64_t r0 = 0; r0 < N; r0 += band) {
-        EntrySpan sp{};
-        sp.i0 = (int)r0;
-        sp.ni = (int)std::min<int64_t>(band, N - r0);
-        sp.j0 = 0;
-        sp.nj = (int)N;
-        sp.base = r0 * N;
-        sp.gs = N * N;
-        sp.is = N;
-        sp.js = 1;
-        spans.push_back(sp);
-    }
-    if (op.prec == RT_PREC_F64) rc = launch_spans<double, double>(op, spans, (double*)op.d_dense, s, err);
-    else rc = launch_spans<float, float>(op, spans, (float*)op.d_dense, s, err);
+    const int rc = op.prec == RT_PREC_F64 ? dense_matrix<double>(op, s, err) : dense_matrix<float>(op, s, err);
     if (rc) return rc;
+    op.info.entries_evaluated += N * N;
     op.info.stored_entries = N * N;
     op.info.apply_bytes = (int64_t)op.F * N * N * (int64_t)esz + 2 * (int64_t)op.F * N * (int64_t)esz;
     op.info.apply_flops = 2 * (int64_t)op.F * N * N;

@@ -113,14 +113,6 @@ struct KernelParams {
     const float4 *tpt, *tcos;  // [4][T] point and weight, cosines
 };
 
-// A rectangular set of entries G_g[i0 + ii][j0 + jj], ii < ni, jj < nj, written
-// to out[base + g*gs + ii*is + jj*js] (float or double, per launch).
-struct EntrySpan {
-    int i0, ni, j0, nj;
-    int64_t base, gs, is, js;
-    int64_t first;   // prefix: index of this span's first entry in the launch
-};
-
 // One far (admissible) block in tree order.
 struct FarBlock {
     int row0, m, col0, n;
@@ -132,7 +124,7 @@ struct ClusterNode {
     int start, size, left, right;
 };
 
-inline int round8(int x) { return (x + 7) & ~7; }
+__host__ __device__ inline int round8(int x) { return (x + 7) & ~7; }
 
 // Leaf chunk of a block's rows: rows [rbeg, rbeg + m) of the block (local),
 // padded to m8 = round8(m), stored at offset off from the block's base.
