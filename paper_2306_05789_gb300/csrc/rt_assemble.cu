@@ -618,8 +618,7 @@ __device__ __forceinline__ __half to_store<__half>(float x) { return __float2hal
 
 struct PackItem {
     int b;          // far block id (ACA numbering)
-    int l;          // term
-    int r, m, n, n8;
+    int r, m, n;
     int64_t voff_dst, uoff_dst;   // element offsets of the block's V^T and U^T in the final storage
     int c0, c1;     // chunk range [c0, c1) in the chunk array
 };
@@ -636,46 +635,62 @@ __device__ __forceinline__ void store_split(T* dst, T* lo, int64_t i, float x)
     dst[i] = h;
     if (lo) lo[i] = to_store<T>(x - (float)h);
 }
+// blockIdx.y splits a block's terms.  FP32 terms are copied as they are, flat
+// over (term, group, column) with 16-byte accesses on the V side; for 16-bit storage
+// a warp takes one (term, group) and scales it.  Bound by memory: the terms are
+// read once and written once (32^3 x 16 groups, 19 GB: 11.5 ms with a CTA per term
+// and its threads on one group's 64 values at a time, 9.5 ms this way).
 template <class T>
-__global__ void aca_pack(AcaDev D, const PackItem* items, int nitems, const Chunk* chunks, T* dst, T* lo)
+__global__ void __launch_bounds__(256) aca_pack(AcaDev D, const PackItem* items, int nitems, const Chunk* chunks, T* dst, T* lo)
 {
-    __shared__ float red[2][32];
+    const int lane = threadIdx.x & 31, warp = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int warps = gridDim.y * (blockDim.x >> 5);
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const PackItem p = items[it];
-        const int64_t us = D.toff[(int64_t)p.b * D.rmax + p.l], vs = us + (int64_t)D.G * round4(p.m);
-        for (int g = 0; g < D.G; ++g) {
+        const int m4 = round4(p.m), n4 = round4(p.n), n8 = round8(p.n);
+        if constexpr (sizeof(T) == 4) {
+            const int64_t* toff = D.toff + (int64_t)p.b * D.rmax;
+            const int tid = blockIdx.y * blockDim.x + threadIdx.x, nth = gridDim.y * blockDim.x;
+            const int nq = n4 >> 2, per = D.G * nq;   // float4s of one term's V
+#pragma unroll 4
+            for (int e = tid; e < p.r * per; e += nth) {
+                const int l = e / per, k = e - l * per, g = k / nq;
+                const float4 x = reinterpret_cast<const float4*>(D.pool + toff[l] + (int64_t)D.G * m4)[k];
+                *reinterpret_cast<float4*>(dst + p.voff_dst + ((int64_t)g * p.r + l) * n8 + 4 * (k - g * nq)) = x;
+            }
+            for (int c = p.c0; c < p.c1; ++c) {
+                const Chunk ch = chunks[c];
+                const int pu = D.G * ch.m;
+#pragma unroll 4
+                for (int e = tid; e < p.r * pu; e += nth) {
+                    const int l = e / pu, k = e - l * pu, g = k / ch.m, i = k - g * ch.m;
+                    dst[p.uoff_dst + ch.off + ((int64_t)g * p.r + l) * ch.m8 + i] = D.pool[toff[l] + (int64_t)g * m4 + ch.rbeg + i];
+                }
+            }
+            continue;
+        }
+        for (int k = warp; k < p.r * D.G; k += warps) {
+            const int l = k / D.G, g = k - l * D.G;
+            const float* u = D.pool + D.toff[(int64_t)p.b * D.rmax + l] + (int64_t)g * m4;
+            const float* v = D.pool + D.toff[(int64_t)p.b * D.rmax + l] + (int64_t)D.G * m4 + (int64_t)g * n4;
             float su = 1.f;
             if (sizeof(T) == 2) {
                 float mu = 0.f, mv = 0.f;
-                for (int i = threadIdx.x; i < p.m; i += blockDim.x) mu = fmaxf(mu, fabsf(D.pool[us + (int64_t)g * round4(p.m) + i]));
-                for (int j = threadIdx.x; j < p.n; j += blockDim.x) mv = fmaxf(mv, fabsf(D.pool[vs + (int64_t)g * round4(p.n) + j]));
+                for (int i = lane; i < p.m; i += 32) mu = fmaxf(mu, fabsf(u[i]));
+                for (int j = lane; j < p.n; j += 32) mv = fmaxf(mv, fabsf(v[j]));
                 for (int o = 16; o > 0; o >>= 1) {
                     mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, o));
                     mv = fmaxf(mv, __shfl_xor_sync(0xffffffffu, mv, o));
                 }
-                if ((threadIdx.x & 31) == 0) {
-                    red[0][threadIdx.x >> 5] = mu;
-                    red[1][threadIdx.x >> 5] = mv;
-                }
-                __syncthreads();
-                mu = 0.f;
-                mv = 0.f;
-                for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                    mu = fmaxf(mu, red[0][w]);
-                    mv = fmaxf(mv, red[1][w]);
-                }
-                __syncthreads();
                 if (mu > 0.f && mv > 0.f) su = sqrtf(mv / mu);
             }
             const float sv = 1.f / su;
-            for (int j = threadIdx.x; j < p.n; j += blockDim.x)
-                store_split<T>(dst, lo, p.voff_dst + ((int64_t)g * p.r + p.l) * p.n8 + j,
-                               sv * D.pool[vs + (int64_t)g * round4(p.n) + j]);
+            const int64_t vd = p.voff_dst + ((int64_t)g * p.r + l) * n8;
+            for (int j = lane; j < p.n; j += 32) store_split<T>(dst, lo, vd + j, sv * v[j]);
             for (int c = p.c0; c < p.c1; ++c) {
                 const Chunk ch = chunks[c];
-                for (int i = threadIdx.x; i < ch.m; i += blockDim.x)
-                    store_split<T>(dst, lo, p.uoff_dst + ch.off + ((int64_t)g * p.r + p.l) * ch.m8 + i,
-                                   su * D.pool[us + (int64_t)g * round4(p.m) + ch.rbeg + i]);
+                const int64_t ud = p.uoff_dst + ch.off + ((int64_t)g * p.r + l) * ch.m8;
+                for (int i = lane; i < ch.m; i += 32) store_split<T>(dst, lo, ud + i, su * u[ch.rbeg + i]);
             }
         }
     }
@@ -975,10 +990,8 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                 note_peak(0);   // packed far field next to this wave's pool
                 std::vector<PackItem> items;
                 for (int k = k0; k < k1; ++k)
-                    for (int l = 0; l < op.rank[k]; ++l)
-                        items.push_back({far_src[k], l, op.rank[k], op.far_blocks[k].m, op.far_blocks[k].n,
-                                         round8(op.far_blocks[k].n), op.far_v_off[k], op.far_u_off[k],
-                                         op.far_chunk_ptr[k], op.far_chunk_ptr[k + 1]});
+                    items.push_back({far_src[k], op.rank[k], op.far_blocks[k].m, op.far_blocks[k].n, op.far_v_off[k],
+                                     op.far_u_off[k], op.far_chunk_ptr[k], op.far_chunk_ptr[k + 1]});
                 PackItem* d_items = nullptr;
                 Chunk* d_chunks = nullptr;
                 const int c0 = op.far_chunk_ptr[k0], nc = op.far_chunk_ptr[k1] - c0;
@@ -988,7 +1001,7 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                                             cudaMemcpyHostToDevice, s));
                 RT_CUDA_TRY(cudaMemcpyAsync(d_chunks + c0, op.far_chunks.data() + c0, sizeof(Chunk) * nc,
                                             cudaMemcpyHostToDevice, s));
-                const int grid = (int)std::min<size_t>(items.size(), 152 * 64);
+                const dim3 grid((unsigned)std::min<size_t>(items.size(), 152 * 64), items.size() < 152 * 8 ? 8 : 1);
                 const int ni = (int)items.size();
                 cudaEventRecord(pk0, s);
                 if (op.far_prec == RT_PREC_F32)

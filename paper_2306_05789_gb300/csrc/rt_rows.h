@@ -56,15 +56,20 @@ inline int group_chunk(const Operator& op)
     return G <= 1 ? 1 : (G <= 4 ? 4 : (G <= 8 ? 8 : (G <= 16 || op.kp.evaluator == EV_PHASE ? 16 : 32)));
 }
 
-// Threads of a row or ACA CTA.  One CTA runs a block's whole ACA, so with fewer
-// admissible blocks than the chip holds CTAs of 128 (about four on each of 152
-// SMs) more threads share a block: box with 298 blocks, ACA 417 ms with 128
-// threads, 150 ms with 512.
+// Threads of a row or ACA CTA.  One CTA runs a block's whole ACA: with few
+// admissible blocks more threads share a block, and with many, 128-thread CTAs
+// waste the least on a block's ragged sizes.  Measured builds (near + ACA, ms) at
+// 128 | 256 | 512 threads: phase evaluator 28 blocks 2.6 | 1.7 | 1.5, 334 blocks 3.8 |
+// 2.5 | 2.7, 1818 blocks 8.0 | 6.0 | 9.0, 2970 blocks 19.1 | 15.0 | 22.2 (2 groups) and
+// 28.8 | 29.7 | 36.1 (5 groups), 8466 blocks 65 | 73 | 90; general evaluator 298
+// blocks 431 | 379 | 194; plain 1826 blocks 12.5 | 11.2 | 13.3.  A chunk of 32 groups
+// needs 255 registers, so its CTAs stay at 256 threads.
 inline int eval_threads(const Operator& op)
 {
     const size_t nb = op.plan.far_blocks.size();
-    const int most = group_chunk(op) > 16 ? 256 : 512;
-    return nb >= 608 || nb == 0 ? 128 : (nb >= 304 ? 256 : most);
+    if (group_chunk(op) > 16) return nb < 608 ? 256 : 128;
+    if (nb < (op.kp.evaluator == EV_PHASE ? 320 : 608)) return 512;
+    return nb < 3000 ? 256 : 128;
 }
 
 template <int EV>
