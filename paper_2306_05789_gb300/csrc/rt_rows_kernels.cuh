@@ -50,7 +50,13 @@ __global__ void __launch_bounds__(max_threads(MG, EV), 1) row_items_kernel(Kerne
 template <class T>
 static int table_alloc(Operator& op, T** p, size_t count, std::string& err)
 {
-    RT_CUDA_TRY(cudaMallocAsync((void**)p, std::max<size_t>(count, 1) * sizeof(T), op.stream));
+    *p = nullptr;
+    const cudaError_t e = cudaMallocAsync((void**)p, std::max<size_t>(count, 1) * sizeof(T), op.stream);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        err = std::string("cudaMallocAsync (assembly tables): ") + cudaGetErrorString(e);
+        return RT_ENOMEM;
+    }
     op.eval_tables.push_back((void*)*p);
     op.eval_bytes += (int64_t)(count * sizeof(T));
     return RT_OK;
