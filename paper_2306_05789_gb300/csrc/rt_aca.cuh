@@ -26,7 +26,7 @@
 // Bound: instruction issue of the row and column evaluation.
 // Measured on GB300, the whole ACA of one operator, before (one launch per
 // phase and step) and after: 32^3 x 16 groups 330 -> 248 ms, 41^3 x 1 group 386 ->
-// 291 ms, 13^3 x 3 groups 9.7 -> 6.0 ms.  Six CTAs an SM and loops that are not
+// 291 ms, 13^3 x 3 groups 9.7 -> 6.0 ms (4.0 ms with 256 threads, eval_threads).  Six CTAs an SM and loops that are not
 // unrolled over the points matter: at four CTAs and unrolled, 431 ms at 41^3,
 // with the warps waiting for instructions (2.6 of 7.4 stall cycles an issue).
 #pragma once

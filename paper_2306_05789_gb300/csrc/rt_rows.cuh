@@ -13,11 +13,14 @@
 // loops that neighbouring tetrahedra contend for.
 //
 // Bound: instruction issue (FP32 and the special-function unit); the tables
-// stay in L2.  Measured on GB300, all launches of one operator build, before
-// (positions and four sines per optical depth, shared atomics) and after:
+// stay in L2.  Measured on GB300, all launches of one operator build that still
+// launched ACA step by step, before (positions and four sines per optical
+// depth, shared atomics) and after (rt_aca.cuh has the ACA's figures since):
 //   32^3, 16 groups: rows and near blocks 433 -> 152 ms, columns 148 -> 71 ms
 //   41^3, 1 group:   rows and near blocks 400 -> 185 ms, columns 454 -> 163 ms
 //   box with grid, walls and corners, 1 group (EV_GENERAL): 901 -> 450 ms
+// Near blocks alone now: 66 ms (32^3), 80 ms (41^3, 98 before the point loops were
+// rolled up and six CTAs ran on an SM).
 // Error of a matvec against FP64, every block dense: 1.34e-7 before and after.
 //
 // (tetrahedron, term) pairs whose source point is near (14-point rule) are
