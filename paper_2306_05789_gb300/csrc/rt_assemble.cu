@@ -17,6 +17,7 @@
 
 #include "rt_entry.cuh"
 #include "rt_internal.h"
+#include "rt_pool.h"
 #include "rt_rows.h"
 
 namespace rt {
@@ -740,16 +741,15 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
     const bool split = op.refine && op.far_prec != RT_PREC_F32;
 
     // ---- waves: consecutive runs of far blocks whose ACA terms (estimated at
-    // kWaveRank terms per block) take at most kWaveBytes of FP32 scratch.  Each
+    // kPoolTerms terms per block) take at most kWaveBytes of FP32 scratch.  Each
     // wave is approximated, packed into the far storage and its scratch freed
     // before the next starts, which bounds the assembly's memory peak.
-    constexpr double kWaveRank = 24.0;
     const int64_t kWaveBytes = op.wave_bytes;
     std::vector<int> wave_start(1, 0);
     {
         double acc = 0.0;
         for (int b = 0; b < nfar; ++b) {
-            const double est = 4.0 * G * (double)(farb[b].m + farb[b].n) * kWaveRank;
+            const double est = 4.0 * G * (double)(farb[b].m + farb[b].n) * (double)kPoolTerms;
             if (acc > 0.0 && acc + est > (double)kWaveBytes) {
                 wave_start.push_back(b);
                 acc = 0.0;
@@ -864,9 +864,10 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
             RT_CUDA_TRY(cudaMemcpyAsync(D.used_off, used_off.data(), sizeof(int64_t) * nb, cudaMemcpyHostToDevice, s));
             std::vector<int> h_rank(nb, 0), status(nb, ACA_ACTIVE);
 
-            // term pool of this wave: kWaveRank terms per block, grown if needed
-            pool_cap = 0;
-            for (int b = 0; b < nb; ++b) pool_cap += aca_term_size(G, fw[b].m, fw[b].n) * (int64_t)kWaveRank;
+            // term pool of this wave, grown if needed
+            int64_t one_term = 0;
+            for (int b = 0; b < nb; ++b) one_term += aca_term_size(G, fw[b].m, fw[b].n);
+            pool_cap = pool_first(one_term);
             if (cudaMallocAsync((void**)&pool, sizeof(float) * pool_cap, s) != cudaSuccess) {
                 cleanup();
                 err = "cudaMalloc (ACA pool) failed";
@@ -916,7 +917,7 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                     break;
                 }
                 // the pool ran out: a larger one, and the active blocks go on
-                const int64_t ncap = std::max<int64_t>(pool_cap + pool_cap / 2, pool_cap + need * 8);
+                const int64_t ncap = pool_grown(pool_cap, need);
                 float* np = nullptr;
                 if (cudaMallocAsync((void**)&np, sizeof(float) * ncap, s) != cudaSuccess) {
                     cudaFreeAsync(pool, s);

@@ -10,7 +10,8 @@ namespace rt {
 
 // State of a wave of admissible blocks during ACA (rt_aca.cuh); block b of the
 // wave.  A term of block b: u [G][m4] then v [G][n4] at toff[b][l] of the pool,
-// rows padded with zeros to multiples of four for 16-byte loads.
+// rows padded with zeros to multiples of four for 16-byte loads (a term's offset
+// is a multiple of four too: rt_pool.h).
 __host__ __device__ inline int round4(int x) { return (x + 3) & ~3; }
 inline int64_t aca_term_size(int G, int m, int n) { return (int64_t)G * (round4(m) + round4(n)); }
 enum { ACA_ACTIVE = 0, ACA_DONE = 1, ACA_DENSE = 2 };

@@ -91,3 +91,40 @@ def test_aca_resumes_when_the_term_pool_runs_out(groups):
         got = Y.double().cpu().numpy()[:, rows]
         assert np.linalg.norm(got - ref) < 4e-6 * np.linalg.norm(ref)
         op.free()
+
+
+def _apply(op, X):
+    import torch
+    Xd = torch.tensor(X, device="cuda")
+    Y = torch.empty_like(Xd)
+    op.apply(Xd, Y)
+    return Y.double().cpu().numpy()
+
+
+@pytest.mark.parametrize("groups", [1, 3, 17])
+@pytest.mark.parametrize("one_block_waves", [False, True])
+def test_aca_of_high_rank_grows_the_pool_many_times(groups, one_block_waves):
+    """Touching blocks of 166 to 666 rows at a tolerance below FP32: every block runs to the rank where
+    dense storage is smaller (83 to 332 terms), so the pool, 24 terms a block at first, grows six times
+    in one wave and four to seven with one block to a wave; the terms' 16-byte accesses need every
+    capacity rounded.  All blocks end dense, and the apply is that of the dense matrix."""
+    import paper_2306_05789_gb300 as rt
+    from oracle import oracle as O
+    p = _problem(11, groups, Z0)
+    X = W.rand_vectors((groups, p.N), seed=1).astype(np.float32)
+    rows = np.arange(0, p.N, 7, dtype=np.int32)
+    c, g = np.unique(np.asarray(p.freqs.c), return_inverse=True)
+    ref = np.stack([np.einsum("ij,j->i", np.asarray(O.G_rows(p, rows, c=c))[:, g[f]], X[f].astype(np.float64))
+                    for f in range(groups)])
+    _, blocks, _ = rt.rt_plan(p.xyz, 200, 2.0, rt.RT_ADM_CENTER)
+    far = blocks[blocks[:, 4] == 1].astype(np.int64)
+    op = rt.rt_build_operator(p, rt.hparams(leaf=200, adm=rt.RT_ADM_CENTER, aca_eps=1e-9,
+                                            wave_bytes=1 if one_block_waves else 0))
+    info = op.info()
+    got = _apply(op, X)[:, rows]
+    op.free()
+    assert info["aca_waves"] == (len(far) if one_block_waves else 1)
+    assert info["n_far"] == 0 and info["n_dense_fallback"] == len(far)
+    # (m + n) floats a term and group: what the blocks took, beyond the capacity after five growths by half
+    assert info["entries_evaluated"] - p.N ** 2 > 24 * 1.5 ** 5 * (far[:, 1] + far[:, 3]).sum()
+    assert np.linalg.norm(got - ref) < 2e-6 * np.linalg.norm(ref)
