@@ -281,7 +281,11 @@ __device__ __forceinline__ void phase_reflected(const KernelParams& P, const Pha
     float k = P.k0f;
     if (P.sinprod) {
         const float dv = dp - dq, du = dp + dq;
-        const float t = (P.wc0 - x.c) * rcp_approx(Z);
+        // x' splits the line from the image at t in [0, 1]; t = 0 where x and y lie in the
+        // wall's plane or rounding puts y behind it (wall_point), which also keeps 0 / 0
+        // out: a vertex on the wall sees a tetrahedron that is flat against it in FP32
+        const float h = P.wc0 - x.c;
+        const float t = h * Z > 0.f ? h * rcp_approx(Z) : 0.f;
         const float v1 = fmaf(t, dv, x.v), u1 = fmaf(t, du, x.u);
         const float hv = P.wcos2 * __cosf((float)(2.0 * kPi) * (v1 - rintf(v1)));
         const float hu = P.wcos2 * __cosf((float)(2.0 * kPi) * (u1 - rintf(u1)));

@@ -128,3 +128,29 @@ def test_aca_of_high_rank_grows_the_pool_many_times(groups, one_block_waves):
     # (m + n) floats a term and group: what the blocks took, beyond the capacity after five growths by half
     assert info["entries_evaluated"] - p.N ** 2 > 24 * 1.5 ** 5 * (far[:, 1] + far[:, 3]).sum()
     assert np.linalg.norm(got - ref) < 2e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("scale,wall", [(1.0, X1), (0.6, ((0.6, 0.3, 0.0), (1.0, 0.0, 0.0), 0.7)), (1.0, Z0)])
+def test_tetrahedron_flat_against_a_wall(scale, wall):
+    """A boundary sliver 1e-9 high lies in the wall's plane once rounded to FP32: rows of vertices on the
+    wall have a reflected path of zero height to it, which must not reach the sums as NaN."""
+    import paper_2306_05789_gb300 as rt
+    from oracle import oracle as O
+    p = _problem(6, 1, wall)
+    p.xyz = p.xyz * scale
+    axis = int(np.argmax(np.abs(wall[1])))
+    at = wall[0][axis]
+    face = np.flatnonzero(np.abs(p.xyz[:, axis] - at) < 1e-12)
+    u, v = [d for d in range(3) if d != axis]
+    corner = face[np.argsort(p.xyz[face, u] + p.xyz[face, v])[:3]]   # three vertices at one corner of the face
+    tip = np.array([0.5, 0.3, 0.2]) @ p.xyz[corner]   # on no quadrature point of the sliver
+    tip[axis] = at + (1e-9 if at == 0.0 else -1e-9)
+    p.tet = np.vstack([p.tet, [[*corner, p.N]]]).astype(np.int32)
+    p.xyz = np.vstack([p.xyz, tip])
+    X = W.rand_vectors((1, p.N), seed=1).astype(np.float32)
+    ref = O.DenseOperator(p).apply(X.astype(np.float64))
+    op = rt.rt_build_operator(p, rt.hparams(eta=1e-9))
+    got = _apply(op, X)
+    op.free()
+    assert np.isfinite(got).all()
+    assert np.linalg.norm(got - ref) < 2e-6 * np.linalg.norm(ref)
