@@ -154,3 +154,28 @@ def test_tetrahedron_flat_against_a_wall(scale, wall):
     op.free()
     assert np.isfinite(got).all()
     assert np.linalg.norm(got - ref) < 2e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("groups", [1, 3])
+def test_blocks_of_several_groups_resume_and_stay_compressed(groups):
+    """eps = 1e-6 takes more than 24 terms a block on average here, so the pool grows, blocks of several
+    groups go on in the larger one, and all of them end compressed.  Tolerance: eps for the far field
+    plus 2e-6 for FP32 entries."""
+    import paper_2306_05789_gb300 as rt
+    from oracle import oracle as O
+    p = _problem(14, groups, Z0)
+    X = W.rand_vectors((groups, p.N), seed=1).astype(np.float32)
+    rows = np.arange(0, p.N, 11, dtype=np.int32)
+    c, g = np.unique(np.asarray(p.freqs.c), return_inverse=True)
+    ref = np.stack([np.einsum("ij,j->i", np.asarray(O.G_rows(p, rows, c=c))[:, g[f]], X[f].astype(np.float64))
+                    for f in range(groups)])
+    _, blocks, _ = rt.rt_plan(p.xyz, 180, 2.0)
+    far, near = (blocks[blocks[:, 4] == k].astype(np.int64) for k in (1, 0))
+    op = rt.rt_build_operator(p, rt.hparams(leaf=180, aca_eps=1e-6))
+    info = op.info()
+    got = _apply(op, X)[:, rows]
+    op.free()
+    assert info["n_far"] == len(far) > 0 and info["n_dense_fallback"] == 0
+    used = info["entries_evaluated"] - (near[:, 1] * near[:, 3]).sum()
+    assert used > 24 * (far[:, 1] + far[:, 3]).sum()
+    assert np.linalg.norm(got - ref) < 3e-6 * np.linalg.norm(ref)
