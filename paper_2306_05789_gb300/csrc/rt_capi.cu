@@ -481,10 +481,14 @@ int build(rt::Operator& op, const rt_problem* P, const rt_hparams* H, cudaStream
         kp.c[g] = op.gc[g];
         kp.cf[g] = (float)op.gc[g];
     }
+    // Equally spaced scales share one exponential through the recurrence exp(-c_{g+1}
+    // tau) = exp(-c_g tau) exp(-dc tau), but only in ascending order: descending, it
+    // starts from the smallest value, which underflows (and its factor overflows: 0 x
+    // inf) at depths where the later groups' values are still large.
     kp.c_arith = 0;
     if (op.G >= 3) {
         const double dc = op.gc[1] - op.gc[0];
-        bool arith = dc != 0.0;
+        bool arith = dc > 0.0;
         for (int g = 2; g < op.G && arith; ++g)
             arith = std::fabs(op.gc[g] - (op.gc[0] + g * dc)) <= 1e-12 * std::max(1.0, std::fabs(op.gc[g]));
         if (arith) {

@@ -71,7 +71,7 @@ struct KernelParams {
     int G;              // groups
     double c[kMaxGroups];
     float cf[kMaxGroups];
-    // group scales in arithmetic progression c_g = c_0 + g dc: the FP32 paths
+    // group scales in ascending arithmetic progression c_g = c_0 + g dc: the FP32 paths
     // get exp(-c_g tau) = exp(-c_0 tau) exp(-dc tau)^g by repeated products
     int c_arith;
     float c0f, dcf;

@@ -179,3 +179,36 @@ def test_blocks_of_several_groups_resume_and_stay_compressed(groups):
     used = info["entries_evaluated"] - (near[:, 1] * near[:, 3]).sum()
     assert used > 24 * (far[:, 1] + far[:, 3]).sum()
     assert np.linalg.norm(got - ref) < 3e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("k0,c", [(50.0, (3.0, 2.0, 1.0)), (12.0, tuple(range(8, 0, -1))), (12.0, tuple(range(1, 9))),
+                                  (12.0, tuple(np.linspace(4.0, 0.25, 16)))])
+@pytest.mark.parametrize("wall", [Z0, OBLIQUE])
+def test_equally_spaced_scales_in_either_order_at_large_depth(k0, c, wall):
+    """Equally spaced group scales, ascending and descending, with optical depths up to 90 per unit scale:
+    every group is finite and agrees with the oracle between opposite faces too, where exp(-c tau) of the
+    larger scales is far below the FP32 range.
+
+    Tolerance: an FP32 optical depth is within 1e-6 of its value in relative terms, so a value
+    exp(-c tau) above 1e-30 (c tau < 70) is within 7e-5."""
+    import paper_2306_05789_gb300 as rt
+    from oracle import oracle as O
+    p = _problem(6, len(c), wall, kind="const")
+    p.kappa.k0 = k0
+    p.freqs.c = np.array(c, dtype=np.float64)
+    ref_op = O.DenseOperator(p)
+    X = W.rand_vectors((len(c), p.N), seed=1).astype(np.float32) + np.float32(0.5)
+    far = X * (p.xyz[:, 0] > 0.79)
+    rows = p.xyz[:, 0] < 0.21
+    for eta in (1e-9, 2.0):
+        op = rt.rt_build_operator(p, rt.hparams(eta=eta))
+        for V, on in ((X, np.ones(p.N, dtype=bool)), (far, rows)):
+            ref = ref_op.apply(V.astype(np.float64))[:, on]
+            got = _apply(op, V)[:, on]
+            assert np.isfinite(got).all()
+            if eta > 1:
+                continue
+            for g in range(len(c)):
+                size = np.linalg.norm(ref[g])
+                assert np.linalg.norm(got[g] - ref[g]) <= 7e-5 * size + 1e-30 * p.N, (g, size)
+        op.free()
