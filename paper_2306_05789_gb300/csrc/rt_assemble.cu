@@ -201,8 +201,8 @@ static int grid_for(int64_t warps)
 // evaluated four times); the vertex sums go to scratch [row][vertex slot][g][T]
 // and dense_gather adds each column's in the order of its tetrahedra.
 // Bound: FP64 issue (1/64 of the FP32 rate): for a constant kappa a term is one
-// rsqrt (1/r^2 and r, and the broken path is as long as the line from the image)
-// and one exponential.  12^3, kappa = 1, one wall, 1.2e8 terms: the whole matrix
+// rsqrt (1/r^2 and r; the broken path is as long as the line from the image when
+// the mesh lies inside the wall) and one exponential.  12^3, kappa = 1, one wall, 1.2e8 terms: the whole matrix
 // 117 ms entry by entry, 15.2 ms this way.
 template <class R>
 __device__ __forceinline__ R rsqrt_r(R x);
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kDenseThreads) dense_tets_kernel(KernelParams 
                                b[0] * v[0].z + b[1] * v[1].z + b[2] * v[2].z + b[3] * v[3].z};
             const R r2 = dist2<R>(src, y);
             R w = scale * vol * tet_w<R>(q) * kappa_at<R, XT>(P, y.x, y.y, y.z) * inv4pi, tau;
-            if (!XT && P.kappa_kind == RT_KAPPA_CONST) {
+            if (!XT && P.kappa_kind == RT_KAPPA_CONST && (t == 0 || P.wall_inside)) {
                 const R rs = rsqrt_r<R>(r2);
                 tau = kp_k0<R>(P) * r2 * rs;
                 w *= rs * rs;

@@ -218,6 +218,22 @@ int group_channels(rt::Operator& op, const rt_freqs& Fq, int bins, std::string& 
     return RT_OK;
 }
 
+// Whether the whole mesh lies on the inner side of the first wall, up to the
+// rounding of its side test: every path from the image then crosses the wall's
+// plane between x and y, and the broken path is as long as the line.
+bool inside_first_wall(const rt::KernelParams& kp, const std::vector<double>& xyz)
+{
+    for (size_t k = 0; k < xyz.size(); k += 3) {
+        double side = 0.0, mag = 0.0;
+        for (int d = 0; d < 3; ++d) {
+            side += (xyz[k + d] - kp.wp[d]) * kp.wn[d];
+            mag += (std::fabs(xyz[k + d]) + std::fabs(kp.wp[d])) * std::fabs(kp.wn[d]);
+        }
+        if (!(side <= 8.9e-16 * mag)) return false;   // 4 units of rounding of every term
+    }
+    return true;
+}
+
 // Whether the phase evaluator (rt_phase.cuh) serves the problem, and its
 // parameters: no further walls, grid or boxes; the first wall, if any, normal
 // to an axis with the whole mesh on its inner side; for the sin-product kappa
@@ -532,6 +548,7 @@ int build(rt::Operator& op, const rt_problem* P, const rt_hparams* H, cudaStream
         kp.cl[g] = (float)l;
         kp.clo[g] = (float)(l - kp.cl[g]);
     }
+    kp.wall_inside = kp.has_wall && inside_first_wall(kp, xyz64) ? 1 : 0;
     phase_setup(op, xyz64);
     kp.xyz32 = op.d_xyz32;
     kp.xyz64 = op.d_xyz64;

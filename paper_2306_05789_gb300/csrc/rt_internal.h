@@ -98,6 +98,7 @@ struct KernelParams {
     // coordinates (p, q, c: the first wall's axis last) and phase cosines
     int evaluator;      // EV_PHASE, EV_PLAIN or EV_GENERAL (rt_rows.cuh)
     int sinprod;        // kappa_kind == RT_KAPPA_SINPROD
+    int wall_inside;    // every vertex on the first wall's inner side
     int axis[3];        // p, q, c as coordinate indices
     float wc0, wc0x2, wcos2;   // wall position C0 along c, 2 C0, 2 cos(2 pi C0)
     float R0f, amp8pi;  // R0; amp / (8 pi)

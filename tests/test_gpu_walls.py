@@ -199,3 +199,27 @@ def test_too_many_walls_are_rejected():
     with pytest.raises(rt.RtError) as e:
         rt.rt_build_operator(p, rt.hparams())
     assert e.value.code == rt.RT_EINVAL
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("n", [(0.0, 0.0, -1.0), (0.2, -0.1, -1.0)])
+def test_dense_entries_of_a_mesh_that_crosses_the_wall(prec, n):
+    """A plane through the domain is accepted; the reflected path of a point behind it is the broken one
+    of the entry evaluator, not the straight line from the image, in the dense matrix as well."""
+    p = W.cube_problem(5, W.Kappa(W.KAPPA_CONST, 1.3, 0.0), W.midpoint_freqs(2), R0=0.5)
+    p.wall = W.Wall((0.0, 0.0, 0.4), n, 0.6)
+    f64 = prec == "f64"
+    op = rt.rt_build_operator(p, rt.hparams(mode=rt.RT_MODE_DENSE, prec=rt.RT_PREC_F64 if f64 else rt.RT_PREC_F32))
+    N = p.N
+    ids = torch.arange(N * N, dtype=torch.int32, device="cuda")
+    want = torch.empty(2, N, N, dtype=torch.float64, device="cuda")
+    for g in range(2):
+        op.eval_entries(g, ids // N, ids % N, want[g])
+    X = torch.rand(2, N, dtype=torch.float64 if f64 else torch.float32, device="cuda")
+    Y = torch.empty_like(X)
+    op.apply(X, Y)
+    ref = torch.einsum("gij,gj->gi", want, X.double())
+    err = float((Y.double() - ref).norm() / ref.norm())
+    op.free()
+    # sums of positive terms, each within about ten roundings on either side
+    assert err < (1e-14 if f64 else 2e-6)
