@@ -202,19 +202,35 @@ static int grid_for(int64_t warps)
 // and dense_gather adds each column's in the order of its tetrahedra.
 // Bound: FP64 issue (1/64 of the FP32 rate): for a constant kappa a term is one
 // rsqrt (1/r^2 and r; the broken path is as long as the line from the image when
-// the mesh lies inside the wall) and one exponential.  12^3, kappa = 1, one wall, 1.2e8 terms: the whole matrix
-// 117 ms entry by entry, 15.2 ms this way.
+// the mesh lies inside the wall) and one exponential.  12^3, kappa = 1, one wall,
+// 1.2e8 terms: the whole matrix 117 ms entry by entry, 15.3 ms this way.
+// Accuracy: the entry evaluator spreads an entry's points over 32 lanes, so the sums
+// here are split too (FP64: per term, and a column's tetrahedra over eight) or
+// compensated (FP32).  Root mean square error of an entry against extended precision,
+// 5^3, oblique wall: FP64 2.03e-16 (entry evaluator 2.03e-16, serial sums 2.20e-16),
+// FP32 1.17e-7 (1.16e-7; serial sums, rsqrt and one weight a point 1.40e-7).
+// A sum of many terms: FP32 compensated (Kahan), FP64 plain
 template <class R>
-__device__ __forceinline__ R rsqrt_r(R x);
-template <>
-__device__ __forceinline__ float rsqrt_r<float>(float x) { return rsqrtf(x); }
-template <>
-__device__ __forceinline__ double rsqrt_r<double>(double x) { return rsqrt(x); }
+struct Sum {
+    R v = R(0), lost = R(0);
+    __device__ __forceinline__ void add(R x)
+    {
+        if constexpr (sizeof(R) == 4) {
+            const R y = x - lost, t = v + y;
+            lost = (t - v) - y;
+            v = t;
+        } else {
+            v += x;
+        }
+    }
+};
 
 constexpr int kDenseThreads = 128;
 template <class R, int MG, bool XT>
 __global__ void __launch_bounds__(kDenseThreads) dense_tets_kernel(KernelParams P, int row0, int g0, R* __restrict__ scratch)
 {
+    // FP64 sums every term of up to four groups by itself (registers for more would spill)
+    constexpr bool by_term = sizeof(R) == 8 && MG <= 4;
     const int tet = blockIdx.x * kDenseThreads + threadIdx.x;
     if (tet >= P.T) return;
     const Vec3<R> xi = load_xyz<R>(P, row0 + blockIdx.y);
@@ -226,11 +242,7 @@ __global__ void __launch_bounds__(kDenseThreads) dense_tets_kernel(KernelParams 
     R diam, vol;
     load_tgeo<R>(P, tet, cen, diam, vol);
     const R lim = R(4) * diam * diam, inv4pi = R(1.0 / (4.0 * kPi));
-    R acc[4][MG];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int g = 0; g < MG; ++g) acc[k][g] = R(0);
+    Sum<R> acc[4][MG];
     const int nt = XT ? 2 + P.n_extra : 2;
     for (int t = 0; t < nt; ++t) {
         if (t == 1 && !P.has_wall) continue;
@@ -239,18 +251,16 @@ __global__ void __launch_bounds__(kDenseThreads) dense_tets_kernel(KernelParams 
         term_source<R>(P, t, xi, xb, src, scale);
         const bool near = dist2<R>(src, cen) < lim;
         const int q0 = near ? 4 : 0, nq = near ? 14 : 4;
+        Sum<R> part[by_term ? 4 : 1][MG];
         for (int q = q0; q < q0 + nq; ++q) {
             const R b[4] = {tet_b<R>(q, 0), tet_b<R>(q, 1), tet_b<R>(q, 2), tet_b<R>(q, 3)};
             const Vec3<R> y = {b[0] * v[0].x + b[1] * v[1].x + b[2] * v[2].x + b[3] * v[3].x,
                                b[0] * v[0].y + b[1] * v[1].y + b[2] * v[2].y + b[3] * v[3].y,
                                b[0] * v[0].z + b[1] * v[1].z + b[2] * v[2].z + b[3] * v[3].z};
-            const R r2 = dist2<R>(src, y);
-            R w = scale * vol * tet_w<R>(q) * kappa_at<R, XT>(P, y.x, y.y, y.z) * inv4pi, tau;
-            if (!XT && P.kappa_kind == RT_KAPPA_CONST && (t == 0 || P.wall_inside)) {
-                const R rs = rsqrt_r<R>(r2);
-                tau = kp_k0<R>(P) * r2 * rs;
-                w *= rs * rs;
-            } else {
+            const R r2 = dist2<R>(src, y), kap = kappa_at<R, XT>(P, y.x, y.y, y.z);
+            const bool straight = !XT && P.kappa_kind == RT_KAPPA_CONST && (t == 0 || P.wall_inside);
+            R w[4], tau;
+            if (!straight) {
                 if constexpr (XT) {
                     tau = term_depth<R>(P, t, xi, src, y);
                     if (!(tau < R(INFINITY))) continue;   // path through an opaque box
@@ -260,23 +270,47 @@ __global__ void __launch_bounds__(kDenseThreads) dense_tets_kernel(KernelParams 
                     const Vec3<R> xp = wall_point<R>(P, src, y);
                     tau = optical_depth<R>(P, xi, xp) + optical_depth<R>(P, xp, y);
                 }
-                w /= r2;
+            }
+            if constexpr (sizeof(R) == 4) {
+                // every hat function's weight as its own product and division: their
+                // roundings differ from vertex to vertex and average out
+                if (straight) tau = kp_k0<R>(P) * sqrt_r(r2);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) w[k] = vol * tet_w<R>(q) * b[k] * kap * inv4pi / r2 * scale;
+            } else {
+                w[0] = scale * vol * tet_w<R>(q) * kap * inv4pi;
+                if (straight) {
+                    const R rs = rsqrt(r2);
+                    tau = kp_k0<R>(P) * r2 * rs;
+                    w[0] *= rs * rs;
+                } else {
+                    w[0] /= r2;
+                }
             }
 #pragma unroll
             for (int g = 0; g < MG; ++g)
                 if (g0 + g < P.G) {
-                    const R cg = kp_c<R>(P, g0 + g);
-                    const R e = w * cg * exp_r(-cg * tau);
+                    const R cg = kp_c<R>(P, g0 + g), E = exp_r(-cg * tau);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[k][g] += b[k] * e;
+                    for (int k = 0; k < 4; ++k) {
+                        Sum<R>& s = by_term ? part[by_term ? k : 0][g] : acc[k][g];
+                        if constexpr (sizeof(R) == 4) s.add(w[k] * cg * E);
+                        else s.v += b[k] * (w[0] * cg * E);
+                    }
                 }
+        }
+        if constexpr (by_term) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int g = 0; g < MG; ++g) acc[k][g].v += part[k][g].v;
         }
     }
     const int64_t row = (int64_t)blockIdx.y * 4 * MG;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int g = 0; g < MG; ++g) scratch[(row + k * MG + g) * P.T + tet] = acc[k][g];
+        for (int g = 0; g < MG; ++g) scratch[(row + k * MG + g) * P.T + tet] = acc[k][g].v;
 }
 
 template <class R, int MG>
@@ -287,13 +321,18 @@ __global__ void __launch_bounds__(256) dense_gather(KernelParams P, int row0, in
     const int t0 = P.vt_ptr[j], t1 = P.vt_ptr[j + 1];
     const int64_t row = (int64_t)blockIdx.y * 4 * MG;
     for (int g = 0; g < MG && g0 + g < P.G; ++g) {
-        R s = R(0);
-#pragma unroll 4
-        for (int e = t0; e < t1; ++e) {
-            const int packed = P.vt_idx[e];
-            s += scratch[(row + (packed & 3) * MG + g) * P.T + (packed >> 2)];
-        }
-        out[(int64_t)(g0 + g) * P.N * P.N + (int64_t)(row0 + blockIdx.y) * P.N + j] = s;
+        // eight partial sums, as the lanes of the entry evaluator keep them: one serial sum of
+        // a column's 24 tetrahedra adds up more rounding than everything before it
+        Sum<R> s[8];
+        for (int e0 = t0; e0 < t1; e0 += 8)
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (e0 + k < t1) {
+                    const int packed = P.vt_idx[e0 + k];
+                    s[k].add(scratch[(row + (packed & 3) * MG + g) * P.T + (packed >> 2)]);
+                }
+        const R all = ((s[0].v + s[1].v) + (s[2].v + s[3].v)) + ((s[4].v + s[5].v) + (s[6].v + s[7].v));
+        out[(int64_t)(g0 + g) * P.N * P.N + (int64_t)(row0 + blockIdx.y) * P.N + j] = all;
     }
 }
 
@@ -331,6 +370,7 @@ static int dense_matrix(Operator& op, cudaStream_t s, std::string& err)
     op.d_dense = d;
     if (op.G <= 1) return dense_rows<R, 1>(op, d, s, err);
     if (op.G <= 4) return dense_rows<R, 4>(op, d, s, err);
+    if (op.G <= 8) return dense_rows<R, 8>(op, d, s, err);   // 11^3, 8 groups: FP32 4.4 -> 2.3 ms, FP64 47 -> 41 ms
     return dense_rows<R, 16>(op, d, s, err);
 }
 

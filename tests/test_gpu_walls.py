@@ -223,3 +223,61 @@ def test_dense_entries_of_a_mesh_that_crosses_the_wall(prec, n):
     op.free()
     # sums of positive terms, each within about ten roundings on either side
     assert err < (1e-14 if f64 else 2e-6)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("wall", [((0.0, 0.0, 0.0), (0.0, 0.0, -1.0), 1.0), ((0.0, 0.0, 0.0), (-0.3, -0.2, -1.0), 1.0)])
+def test_dense_entries_are_as_accurate_as_the_entry_evaluator(prec, wall):
+    """Constant kappa: the dense matrix against an extended-precision sum over the same quadrature points
+    is no further off than rt_eval_entries, which takes an IEEE root and division a point (4 % for the
+    different order of the sums)."""
+    L = np.longdouble
+    f64 = prec == "f64"
+    p = W.cube_problem(5, W.Kappa(W.KAPPA_CONST, 1.3, 0.0), W.midpoint_freqs(1), R0=0.0)
+    inner = ((p.xyz > 1e-9) & (p.xyz < 1 - 1e-9)).all(axis=1)
+    p.xyz[inner] += np.random.default_rng(3).uniform(-0.03, 0.03, size=(int(inner.sum()), 3))
+    p.wall = W.Wall(*wall)
+    N, c, k0 = p.N, L(p.freqs.c[0]), L(1.3)
+    four_pi = 4 * (L(np.pi) + L(1.2246467991473532e-16))
+    x = p.xyz.astype(L)
+    n = np.array(wall[1], dtype=np.float64)
+    n = (n / np.sqrt((n * n).sum())).astype(L)
+    V = x[p.tet]
+    e = V[:, 1:] - V[:, :1]
+    vol = np.abs((e[:, 0] * np.cross(e[:, 1], e[:, 2])).sum(-1)) / 6
+    cen = V.mean(axis=1)
+    lim = 4 * np.max([((V[:, i] - V[:, j]) ** 2).sum(-1) for i in range(4) for j in range(i)], axis=0)
+    al, be = (5 + 3 * np.sqrt(L(5))) / 20, (5 - np.sqrt(L(5))) / 20
+    far_rule = [([al if d == k else be for d in range(4)], L(1) / 4) for k in range(4)]
+    near_rule = []
+    for s, w in ((0.0927352503108912, 0.07349304311636196), (0.3108859192633006, 0.1126879257180159)):
+        near_rule += [([1 - 3 * L(s) if d == k else L(s) for d in range(4)], L(w)) for k in range(4)]
+    s = L(0.4544962958743504)
+    near_rule += [([s if d in (a, b) else L(0.5) - s for d in range(4)], L(0.04254602077708147))
+                  for a in range(4) for b in range(a + 1, 4)]
+    G = np.zeros((N, N), dtype=L)
+    for i in range(N):
+        for src in (x[i], x[i] - 2 * (x[i] @ n) * n):
+            near = ((src - cen) ** 2).sum(-1) < lim
+            for rule, use in ((far_rule, ~near), (near_rule, near)):
+                t = np.flatnonzero(use)
+                for b, w in rule:
+                    b = np.array(b, dtype=L)
+                    r2 = ((src - np.einsum("k,tkd->td", b, V[t])) ** 2).sum(-1)
+                    v = vol[t] * w * k0 * c / four_pi / r2 * np.exp(-c * k0 * np.sqrt(r2))
+                    np.add.at(G[i], p.tet[t].ravel(), (v[:, None] * b).ravel())
+    op = rt.rt_build_operator(p, rt.hparams(mode=rt.RT_MODE_DENSE, prec=rt.RT_PREC_F64 if f64 else rt.RT_PREC_F32))
+    dense = np.empty((N, N))
+    X = torch.zeros(1, N, dtype=torch.float64 if f64 else torch.float32, device="cuda")
+    Y = torch.empty_like(X)
+    for j in range(N):
+        X.zero_()
+        X[0, j] = 1
+        op.apply(X, Y)
+        dense[:, j] = Y[0].double().cpu().numpy()
+    ids = torch.arange(N * N, dtype=torch.int32, device="cuda")
+    each = torch.empty(N, N, dtype=torch.float64, device="cuda")
+    op.eval_entries(0, ids // N, ids % N, each)
+    op.free()
+    rms = [float(np.sqrt((((M - G) / G) ** 2).mean())) for M in (dense, each.cpu().numpy())]
+    assert rms[0] <= 1.04 * rms[1], rms
