@@ -121,7 +121,13 @@ int assemble_setup_constants(Operator& op, std::string& err)
         op.kp.gu32[g] = (float)u;
         op.kp.gw32[g] = (float)hw;
     }
-    return upload_rules(err);
+    // every unit at the first build, whichever of them it needs: the uploads wait for the
+    // device, which a later build must not do while another thread captures a solve
+    int rc;
+    if ((rc = upload_rules(err))) return rc;
+    if ((rc = RowEval<EV_PHASE>::setup(err))) return rc;
+    if ((rc = RowEval<EV_PLAIN>::setup(err))) return rc;
+    return RowEval<EV_GENERAL>::setup(err);
 }
 
 // ---------------------------------------------------------------------------

@@ -75,6 +75,8 @@ inline int eval_threads(const Operator& op)
 
 template <int EV>
 struct RowEval {
+    // what this unit needs once per device: its quadrature rules, its kernels' shared memory
+    static int setup(std::string& err);
     // device tables (sub-clusters, gather lists, point tables) for the sub-clusters' tetrahedra
     static int tables(Operator& op, const std::vector<int>& tets, std::string& err);
     // rows of device items; sums: most (rows x columns) of one item

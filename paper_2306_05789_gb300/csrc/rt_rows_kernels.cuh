@@ -45,6 +45,33 @@ __global__ void __launch_bounds__(max_threads(MG, EV), 1) row_items_kernel(Kerne
         else if constexpr (EV != EV_PHASE) MACRO(32, EV); \
     } while (0)
 
+template <int EV>
+int RowEval<EV>::setup(std::string& err)
+{
+    const int rc = upload_rules(err);
+    if (rc) return rc;
+    static bool attr_set[64] = {false};
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 64 && !attr_set[dev]) {
+#define RT_ROW_ATTR(MG, EV) \
+    RT_CUDA_TRY(cudaFuncSetAttribute(row_items_kernel<MG, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)); \
+    RT_CUDA_TRY(cudaFuncSetAttribute(aca_block_kernel<MG, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024))
+        RT_ROW_ATTR(1, EV);
+        RT_ROW_ATTR(4, EV);
+        RT_ROW_ATTR(8, EV);
+        RT_ROW_ATTR(16, EV);
+        if constexpr (EV != EV_PHASE) {
+            RT_ROW_ATTR(32, EV);
+        }
+#undef RT_ROW_ATTR
+        attr_set[dev] = true;
+    }
+    return RT_OK;
+}
+
 // Device tables of the row and column evaluation: sub-clusters, gather lists,
 // point tables (rt_rows.cuh, rt_phase.cuh).  They live until the assembly ends.
 template <class T>
@@ -67,9 +94,8 @@ int RowEval<EV>::tables(Operator& op, const std::vector<int>& tets, std::string&
 {
     int rc;
     cudaStream_t s = op.stream;
-    if ((rc = upload_rules(err))) return rc;
     int pt = 0;
-const int nth = eval_threads(op);
+    const int nth = eval_threads(op);
 #define RT_PASS_TETS(MG, EV) pt = RowShape<MG, EV>::TPT * nth
     RT_DISPATCH_MG(op, RT_PASS_TETS);
 #undef RT_PASS_TETS
@@ -119,25 +145,6 @@ const int nth = eval_threads(op);
 #undef RT_PASS_LISTS
     }
     RT_CUDA_TRY(cudaGetLastError());
-    static bool attr_set[64] = {false};
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 64 && !attr_set[dev]) {
-#define RT_ROW_ATTR(MG, EV) \
-    RT_CUDA_TRY(cudaFuncSetAttribute(row_items_kernel<MG, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)); \
-    RT_CUDA_TRY(cudaFuncSetAttribute(aca_block_kernel<MG, EV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024))
-        RT_ROW_ATTR(1, EV);
-        RT_ROW_ATTR(4, EV);
-        RT_ROW_ATTR(8, EV);
-        RT_ROW_ATTR(16, EV);
-        if constexpr (EV != EV_PHASE) {
-            RT_ROW_ATTR(32, EV);
-        }
-#undef RT_ROW_ATTR
-        attr_set[dev] = true;
-    }
     return RT_OK;
 }
 

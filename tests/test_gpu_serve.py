@@ -9,6 +9,10 @@ far field with high + low refinement sweeps).  The budget is never exceeded.
 """
 from __future__ import annotations
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -21,6 +25,7 @@ import workloads as W
 from oracle import oracle as O
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -153,3 +158,53 @@ def test_served_requests_with_walls_grids_and_opaque_boxes():
     rows = W.sample_rows(koba.N, 24, seed=61)
     r = O.one_step_residual(koba, rows, J.astype(np.float64), T)
     assert np.linalg.norm(r) / np.linalg.norm(J[:, rows]) < 1e-5
+
+
+_CAPTURE = """
+import threading, torch
+import paper_2306_05789_gb300 as rt
+import workloads as W
+phase = W.cube_problem(5, W.sinprod_kappa(0.5), W.midpoint_freqs(2), R0=0.5)
+oblique = W.cube_problem(5, W.sinprod_kappa(0.5), W.midpoint_freqs(2), R0=0.5)
+oblique.wall = W.Wall((0.0, 0.0, 0.0), (-0.3, -0.2, -1.0), 0.5)
+walls = W.cube_problem(5, W.sinprod_kappa(0.5), W.midpoint_freqs(2), R0=0.5)
+walls.more_walls = (W.wall_y0(0.4),)
+rt.rt_build_operator(phase, rt.hparams(leaf=16)).free()
+out = []
+def build(p):
+    try:
+        s = torch.cuda.Stream()
+        op = rt.rt_build_operator(p, rt.hparams(leaf=16), stream=s)
+        out.append(op)
+    except Exception as e:
+        out.append(e)
+x = torch.ones(16, device="cuda")
+y = torch.empty_like(x)
+s = torch.cuda.Stream()
+torch.cuda.synchronize()
+for p in (oblique, walls):
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s):
+        g.capture_begin(capture_error_mode="thread_local")
+        torch.add(x, 1.0, out=y)
+        t = threading.Thread(target=build, args=(p,))
+        t.start()
+        t.join()
+        torch.mul(y, 2.0, out=y)
+        g.capture_end()
+    g.replay()
+    torch.cuda.synchronize()
+    assert float(y.sum()) == 64.0
+assert all(isinstance(o, rt.Operator) for o in out), out
+for o in out:
+    o.free()
+print("ok")
+"""
+
+
+def test_first_build_of_an_evaluator_leaves_another_threads_capture_alone():
+    """Solves record their iterations in a graph while other requests build.  What a build uploads once
+    per process must be on the device after the first build, of whatever kind: an upload that waits
+    for the device is not allowed while a stream is being captured."""
+    r = subprocess.run([sys.executable, "-c", _CAPTURE], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
