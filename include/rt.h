@@ -218,7 +218,7 @@ typedef struct {
     int64_t apply_flops;
     int64_t device_bytes;        /* device memory held by the operator */
     double ms_tree, ms_near, ms_aca, ms_pack, ms_source; /* assembly phase times */
-    int64_t peak_bytes;          /* largest device footprint during assembly (operator + ACA scratch) */
+    int64_t peak_bytes;          /* largest device footprint during assembly (operator, ACA scratch, evaluation tables) */
     int64_t aca_waves;           /* waves of admissible blocks the ACA ran in */
     int64_t apply_tensor_cores;  /* 1 if rt_apply runs on the tcgen05 multi-right-hand-side path */
     int64_t assembly_terms;      /* H-matrix assembly: kernel terms evaluated (one direct or one reflected

@@ -569,6 +569,62 @@ void eval_tables_free(Operator& op)
     op.kp.pxyz = op.kp.pcos = op.kp.tcen = op.kp.tpt = op.kp.tcos = nullptr;
 }
 
+// a column cluster's sub-clusters: the nodes of at most kSubCols columns below it, in
+// order; false where a leaf is wider
+static bool sub_clusters(const Plan& P, int cluster, std::vector<int>& out)
+{
+    std::vector<int> stack = {cluster};
+    while (!stack.empty()) {
+        const int k = stack.back();
+        stack.pop_back();
+        const ClusterNode& C = P.clusters[k];
+        if (C.size <= kSubCols) {
+            out.push_back(k);
+        } else if (C.left < 0) {
+            return false;
+        } else {
+            stack.push_back(C.right);
+            stack.push_back(C.left);
+        }
+    }
+    return true;
+}
+
+static std::vector<char> column_clusters(const Plan& P)
+{
+    std::vector<char> used(P.clusters.size(), 0);
+    for (const FarBlock& b : P.far_blocks) used[b.sc] = 1;
+    for (const FarBlock& b : P.near_blocks) used[b.sc] = 1;
+    return used;
+}
+
+int64_t eval_bytes_bound(const Plan& P, int64_t T, int G, int ev)
+{
+    const int mg = group_chunk(G, ev);
+    const int64_t pt = (int64_t)tets_per_thread(mg, ev) * eval_threads(G, ev, P.far_blocks.size());
+    int64_t bytes = T * (ev == EV_PHASE ? 144 : 80) + (ev == EV_PHASE ? (int64_t)P.N * 32 : 0);
+    const std::vector<char> used = column_clusters(P);
+    std::vector<char> seen(P.clusters.size(), 0);
+    std::vector<int> sub;
+    for (int c = 0; c < (int)P.clusters.size(); ++c) {
+        if (!used[c]) continue;
+        sub.clear();
+        sub_clusters(P, c, sub);
+        for (int k : sub) {
+            if (seen[k]) continue;
+            seen[k] = 1;
+            const int64_t pairs = std::min<int64_t>(T, (int64_t)(4.0 * (double)T / P.N * P.clusters[k].size) + 1);
+            const int64_t passes = (pairs + pt - 1) / pt;
+            bytes += (int64_t)sizeof(SubInfo) + 4 * pairs + passes * (8 * pt + 4 * kRunWords + 4);
+        }
+    }
+    for (const FarBlock& b : P.near_blocks) {
+        const int rows = rows_per_item(mg, std::min(b.n, kSubCols));
+        bytes += (int64_t)((b.m + rows - 1) / rows + 1) * (int64_t)sizeof(RowItem);
+    }
+    return bytes;
+}
+
 // sub-clusters of every column cluster and the tetrahedra touching each
 int prepare_row_eval(Operator& op, std::string& err)
 {
@@ -580,29 +636,13 @@ int prepare_row_eval(Operator& op, std::string& err)
     op.sub_size.clear();
     op.sub_tet_ptr.assign(1, 0);
     std::vector<int> sub_id(nc, -1), tets, stamp(op.T, -1);
-    std::vector<char> used(nc, 0);
-    for (const FarBlock& b : P.far_blocks) used[b.sc] = 1;
-    for (const FarBlock& b : P.near_blocks) used[b.sc] = 1;
+    const std::vector<char> used = column_clusters(P);
     std::vector<std::vector<int>> subs(nc);
-    for (int c = 0; c < nc; ++c) {
-        if (!used[c]) continue;
-        std::vector<int> stack = {c};
-        while (!stack.empty()) {
-            const int k = stack.back();
-            stack.pop_back();
-            const ClusterNode& C = P.clusters[k];
-            if (C.size <= kSubCols || C.left < 0) {
-                if (C.size > kSubCols) {
-                    err = "cluster leaf larger than the row-evaluation width";
-                    return RT_EINVAL;
-                }
-                subs[c].push_back(k);
-            } else {
-                stack.push_back(C.right);
-                stack.push_back(C.left);
-            }
+    for (int c = 0; c < nc; ++c)
+        if (used[c] && !sub_clusters(P, c, subs[c])) {
+            err = "cluster leaf larger than the row-evaluation width";
+            return RT_EINVAL;
         }
-    }
     for (int c = 0; c < nc; ++c) {
         for (int k : subs[c]) {
             if (sub_id[k] < 0) {
@@ -626,10 +666,6 @@ int prepare_row_eval(Operator& op, std::string& err)
     }
     return RT_EVALUATOR(op, tables(op, tets, err));
 }
-
-// rows of one item: the more, the wider the stores of a column's rows; the sums
-// of all its rows take at most 8 KB, which keeps four CTAs on an SM at 16 groups
-static int rows_per_item(int mg, int n) { return std::max(1, std::min(8, 8192 / (4 * mg * n))); }
 
 static int launch_rows(Operator& op, const std::vector<RowItem>& items, float* out, cudaStream_t s, std::string& err)
 {
@@ -1121,6 +1157,7 @@ int assemble_hmatrix(Operator& op, cudaStream_t s, std::string& err)
                 }
             }
         }
+        note_peak((int64_t)(sizeof(RowItem) * ritems.size()));   // near blocks, tables and items
         if ((rc = launch_rows(op, ritems, op.d_near, s, err))) return rc;
         for (int k = 0; k < op.n_near; ++k)
             op.info.entries_evaluated += (int64_t)op.dense_blocks[k].m * op.dense_blocks[k].n;

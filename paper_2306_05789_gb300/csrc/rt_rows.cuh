@@ -51,8 +51,6 @@ constexpr int nth = 128;
 // CTAs of the row and ACA kernels on an SM, by registers (16 groups: also by shared memory)
 constexpr int ctas_per_sm(int mg, int ev) { return ev != EV_PHASE ? (mg <= 16 ? 4 : 2) : (mg <= 4 ? 6 : (mg <= 8 ? 5 : 4)); }
 
-constexpr int kRunWords = kSubCols + 4;   // per pass: run count, runs, end mark
-
 // Threads of a row or ACA kernel's CTA are a launch parameter: 128, or more when
 // a problem has too few blocks to fill the chip (eval_threads in rt_rows.h).
 // max_threads is the most that the registers of an instance allow; 128-thread
@@ -64,7 +62,7 @@ constexpr int max_threads(int mg, int ev) { return ev != EV_PHASE ? (mg <= 16 ? 
 // tetrahedron padded so that its 16-byte stores fall into different banks.
 template <int MG, int EV>
 struct RowShape {
-    static constexpr int TPT = MG == 1 && EV == EV_PHASE ? 4 : 1;
+    static constexpr int TPT = tets_per_thread(MG, EV);
     static constexpr int RS = MG == 1 ? 4 : 4 * MG + 4;
     static constexpr int TERMS = EV == EV_GENERAL ? 2 + kMaxXTerms : 2;   // most list entries per tetrahedron
     static __host__ __device__ constexpr int list(int nt) { return 2 * TERMS * TPT * nt; }   // two passes

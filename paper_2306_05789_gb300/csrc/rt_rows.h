@@ -4,6 +4,8 @@
 // instances compile in parallel.
 #pragma once
 
+#include <algorithm>
+
 #include "rt_internal.h"
 
 namespace rt {
@@ -51,11 +53,11 @@ struct SubInfo {
 // cost about as much as 16 groups' exponentials and sums, and its chunks of 16
 // keep four CTAs on an SM; the others' terms cost several times that, so they
 // take up to 32 groups at once.
-inline int group_chunk(const Operator& op)
+inline int group_chunk(int G, int ev)
 {
-    const int G = op.G;
-    return G <= 1 ? 1 : (G <= 4 ? 4 : (G <= 8 ? 8 : (G <= 16 || op.kp.evaluator == EV_PHASE ? 16 : 32)));
+    return G <= 1 ? 1 : (G <= 4 ? 4 : (G <= 8 ? 8 : (G <= 16 || ev == EV_PHASE ? 16 : 32)));
 }
+inline int group_chunk(const Operator& op) { return group_chunk(op.G, op.kp.evaluator); }
 
 // Threads of a row or ACA CTA.  One CTA runs a block's whole ACA: with few
 // admissible blocks more threads share a block, and with many, 128-thread CTAs
@@ -65,13 +67,26 @@ inline int group_chunk(const Operator& op)
 // 28.8 | 29.7 | 36.1 (5 groups), 8466 blocks 65 | 73 | 90; general evaluator 298
 // blocks 431 | 379 | 194; plain 1826 blocks 12.5 | 11.2 | 13.3.  A chunk of 32 groups
 // needs 255 registers, so its CTAs stay at 256 threads.
-inline int eval_threads(const Operator& op)
+inline int eval_threads(int G, int ev, size_t nb)
 {
-    const size_t nb = op.plan.far_blocks.size();
-    if (group_chunk(op) > 16) return nb < 608 ? 256 : 128;
-    if (nb < (op.kp.evaluator == EV_PHASE ? 320 : 608)) return 512;
+    if (group_chunk(G, ev) > 16) return nb < 608 ? 256 : 128;
+    if (nb < (ev == EV_PHASE ? 320 : 608)) return 512;
     return nb < 3000 ? 256 : 128;
 }
+inline int eval_threads(const Operator& op) { return eval_threads(op.G, op.kp.evaluator, op.plan.far_blocks.size()); }
+
+constexpr int kRunWords = kSubCols + 4;   // per pass: run count, runs, end mark
+constexpr int tets_per_thread(int mg, int ev) { return mg == 1 && ev == EV_PHASE ? 4 : 1; }
+
+// rows of one near-block item: the more, the wider the stores of a column's rows; the
+// sums of all its rows take at most 8 KB, which keeps four CTAs on an SM at 16 groups
+inline int rows_per_item(int mg, int n) { return std::max(1, std::min(8, 8192 / (4 * mg * n))); }
+
+// Device bytes of the tables and near-block items that live until the near blocks are
+// done (RowEval::tables, launch_rows), before anything is built: a sub-cluster of k
+// vertices touches at most the sum of its vertices' tetrahedra (about half of it on a
+// Kuhn mesh, whose tetrahedra share vertices).
+int64_t eval_bytes_bound(const Plan& P, int64_t T, int G, int ev);
 
 template <int EV>
 struct RowEval {

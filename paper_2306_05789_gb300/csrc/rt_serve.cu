@@ -9,7 +9,7 @@
 // copied out; then everything of it is freed in stream order and the budget
 // it held is returned, which may admit the next request.  Builds and solves of
 // different slots run concurrently on the device: the host waits in the
-// assembly (one per ACA sweep) and in the fixed point (one per convergence
+// assembly (one per ACA launch) and in the fixed point (one per convergence
 // check) block only their own slot.
 #include <algorithm>
 #include <chrono>
@@ -24,6 +24,8 @@
 #include <vector>
 
 #include "rt_internal.h"
+#include "rt_pool.h"
+#include "rt_rows.h"
 
 namespace rt {
 
@@ -62,19 +64,21 @@ struct Request {
 // size while the fixed point runs.  Exact for the near field and the vectors;
 // the far field assumes every admissible block reaches rank r_hat, a little
 // above the mean rank that ACA reaches at the given tolerance (about 19 at
-// 1e-4 on the cube workloads).  The ACA term scratch lives one wave at a time
-// (at most hp.wave_bytes of 24-term pools, grown by half once at worst) and
-// is gone before the near field is allocated.
+// 1e-4 on the cube workloads).  The ACA scratch of one wave (at most
+// hp.wave_bytes of 24-term pools; an old and a new pool while one grows) is gone
+// before the near field is allocated; the evaluation tables stay until that is
+// filled.
 struct Footprint {
     int64_t peak = 0, resident = 0;
 };
 
-static Footprint estimate_footprint(const Plan& P, int64_t N, int64_t T, int F, int G, const rt_hparams& hp)
+// ev: the evaluator of the rows
+static Footprint estimate_footprint(const Plan& P, int64_t N, int64_t T, int F, int G, int ev, const rt_hparams& hp)
 {
     const double r_hat = std::max(8.0, 6.0 * std::log10(1.0 / hp.aca_eps));
     const int esz = hp.far_prec == RT_PREC_F32 ? 4 : (hp.refine ? 4 : 2);
     std::vector<Chunk> tmp;
-    int64_t near = 0, far_elems = 0, pool = 0, bufs = 0;
+    int64_t near = 0, far_elems = 0, term = 0, rows = 0;
     for (const FarBlock& b : P.near_blocks) {
         tmp.clear();
         near += block_chunks(P, b.row0, b.m, (int64_t)G * b.n, tmp);
@@ -83,17 +87,29 @@ static Footprint estimate_footprint(const Plan& P, int64_t N, int64_t T, int F, 
         tmp.clear();
         const int64_t mpad = block_chunks(P, b.row0, b.m, 1, tmp);
         far_elems += (int64_t)std::ceil(G * r_hat) * ((int64_t)round8(b.n) + mpad);
-        pool += (int64_t)G * 24 * (b.m + b.n);
-        bufs += (int64_t)G * (b.m + b.n);
+        term += aca_term_size(G, b.m, b.n);
+        rows += b.m;
     }
+    // one wave: its share of the terms, pools until r_hat terms a block fit, block states
     const int64_t wave = hp.wave_bytes > 0 ? hp.wave_bytes : ((int64_t)8 << 30);
-    const int64_t aca = (int64_t)(1.5 * (double)std::min<int64_t>(4 * pool, wave)) +
-                        std::min<int64_t>(4 * bufs, wave / 24 + ((int64_t)64 << 20));
+    const double share = std::min(1.0, (double)wave / std::max(1.0, 4.0 * kPoolTerms * (double)term));
+    const int64_t need = (int64_t)(share * (double)term) + 1;
+    int64_t cap = pool_first(need), pools = cap + cap / 2;
+    while ((double)cap < r_hat * (double)need) {
+        const int64_t next = pool_grown(cap, need);
+        pools = cap + next;
+        cap = next;
+    }
+    const int64_t rank_max = hp.rank_max > 0 ? hp.rank_max : 512;
+    const int64_t state = (int64_t)(share * (double)P.far_blocks.size() + 1.0) * (8 * rank_max + 12 * G + 64) +
+                          (int64_t)(share * (double)rows);
+    const int64_t aca = P.far_blocks.empty() ? 0 : 4 * pools + state;
+    const int64_t tables = eval_bytes_bound(P, T, G, ev);
     const int64_t geo = N * 64 + T * 120 + (int64_t)F * N * 4;
     const int64_t vec = (int64_t)F * N * 4 * 6 + N * 16 + (int64_t)F * (int64_t)P.far_blocks.size() * (int64_t)r_hat * 4;
     Footprint f;
     f.resident = geo + 4 * near + (int64_t)esz * far_elems + vec;
-    f.peak = geo + (int64_t)esz * far_elems + std::max<int64_t>(aca, 4 * near + vec);
+    f.peak = geo + (int64_t)esz * far_elems + std::max({tables + aca, tables + 4 * near, 4 * near + vec});
     return f;
 }
 
@@ -323,7 +339,10 @@ int rt_submit(rt_server* h, const rt_problem* P, int64_t* id)
         std::vector<double> cs;
         for (int64_t f = 0; f < F; ++f)
             if (std::find(cs.begin(), cs.end(), r->c[f]) == cs.end()) cs.push_back(r->c[f]);
-        const rt::Footprint fp = rt::estimate_footprint(r->plan, N, T, (int)F, (int)cs.size(), S.o.hp);
+        // the phase evaluator's tables are the largest: they stand for every plain problem
+        const bool ext = P->n_walls > 1 || P->n_obstacles > 0 || P->kappa.kind == RT_KAPPA_GRID;
+        const int ev = ext ? rt::EV_GENERAL : rt::EV_PHASE;
+        const rt::Footprint fp = rt::estimate_footprint(r->plan, N, T, (int)F, (int)cs.size(), ev, S.o.hp);
         r->est_peak = fp.peak;
         r->est_resident = fp.resident;
         r->info.N = N;

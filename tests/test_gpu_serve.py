@@ -208,3 +208,20 @@ def test_first_build_of_an_evaluator_leaves_another_threads_capture_alone():
     for the device is not allowed while a stream is being captured."""
     r = subprocess.run([sys.executable, "-c", _CAPTURE], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("n,F,kw", [(10, 1, dict(eta=1e-9)), (9, 4, dict(eta=1e-9)), (16, 3, {}),
+                                    (14, 1, dict(leaf=128)), (16, 5, dict(far_prec=rt.RT_PREC_BF16, refine=1)),
+                                    (12, 20, dict(leaf=32)), (16, 2, dict(wave_bytes=1 << 22))])
+@pytest.mark.parametrize("walls", [1, 2])
+def test_a_request_stays_within_its_estimate(n, F, kw, walls):
+    """What a request holds at its assembly's peak, tables included, is within what admission reserved."""
+    p = W.cube_problem(n, W.sinprod_kappa(0.5), W.midpoint_freqs(F), R0=0.5)
+    if walls == 2:
+        p.more_walls = (W.wall_y0(0.4),)
+    res, _ = serve([p], rt.hparams(**kw), slots=1)
+    info = res[0][2]
+    assert info["peak_bytes"] <= info["est_bytes"]
+    if kw.get("eta") == 1e-9:   # near blocks, mesh and tables are on the device together
+        T = p.tet.shape[0]
+        assert info["peak_bytes"] >= 4 * F * p.N ** 2 + (116 + (144 if walls == 1 else 80)) * T
