@@ -280,7 +280,6 @@ struct Operator {
     int* d_sub_tets = nullptr;
     double min_diam = 1e300;                               // smallest tetrahedron diameter
     // tables of the row and column evaluation (rt_rows.cuh); freed when the assembly ends
-    std::vector<int> sub_pass0;                            // first pass of every sub-cluster
     void* d_subs = nullptr;                                // SubInfo [sub-clusters]
     unsigned short* d_pass_ref = nullptr;
     unsigned* d_pass_run = nullptr;

@@ -177,13 +177,6 @@ struct GroupSum {
             d[k] = v;
         }
     }
-    // this += f row_values
-    __device__ __forceinline__ void axpy(float f, const GroupSum& o)
-    {
-        const f32x2 ff = pack2(f, f);
-#pragma unroll
-        for (int h = 0; h < MG / 2; ++h) e[h] = fma2(ff, o.e[h], e[h]);
-    }
     __device__ __forceinline__ float get(int g) const
     {
         float a = 0.f, b = 0.f, r = 0.f;
@@ -208,7 +201,6 @@ struct GroupSum<1> {
     __device__ __forceinline__ void store(float* row) const { row[0] = e; }
     __device__ __forceinline__ void blend(float* row, float b, float g) const { row[0] = fmaf(b, e, g * row[0]); }
     __device__ __forceinline__ void add_to(float* row, float b) const { row[0] = fmaf(b, e, row[0]); }
-    __device__ __forceinline__ void axpy(float f, const GroupSum& o) { e = fmaf(f, o.e, e); }
     __device__ __forceinline__ float get(int) const { return e; }
 };
 

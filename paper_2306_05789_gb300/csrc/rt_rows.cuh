@@ -7,7 +7,7 @@
 // value at point q reaches vertex q with weight a and the others with b, so a
 // tetrahedron's four vertex sums are b S + (a - b) e_q with S = sum e_q: one
 // addition per point and group instead of four products.  The vertex sums go
-// to shared memory (nth tetrahedra a pass) and every column gathers
+// to shared memory (a pass of tetrahedra at a time) and every column gathers
 // its own from a list made once per operator: plain stores and loads in place
 // of 4 G shared float atomics per tetrahedron, which are compare-and-swap
 // loops that neighbouring tetrahedra contend for.
@@ -46,10 +46,6 @@ __device__ __forceinline__ void count_work(const KernelParams& P, unsigned terms
         atomicAdd(P.work + 1, (unsigned long long)depths);
     }
 }
-
-constexpr int nth = 128;
-// CTAs of the row and ACA kernels on an SM, by registers (16 groups: also by shared memory)
-constexpr int ctas_per_sm(int mg, int ev) { return ev != EV_PHASE ? (mg <= 16 ? 4 : 2) : (mg <= 4 ? 6 : (mg <= 8 ? 5 : 4)); }
 
 // Threads of a row or ACA kernel's CTA are a launch parameter: 128, or more when
 // a problem has too few blocks to fill the chip (eval_threads in rt_rows.h).

@@ -115,8 +115,6 @@ __device__ __forceinline__ double so_sum(double v, double* sd)
     return sd[0];
 }
 
-// ranks[job] = rank reached, or -1 when the block must stay dense.  `used`
-// (scratch, one byte per row of every job) marks the rows already pivoted.
 // x - sum_{q<k} a[q] b[q]; a and b are rows of kRankCap floats, read 16 bytes at a time
 __device__ __forceinline__ float so_residual(float x, const float* a, const float* b, int k)
 {
@@ -133,6 +131,8 @@ __device__ __forceinline__ float so_residual(float x, const float* a, const floa
     return x;
 }
 
+// ranks[job] = rank reached, or -1 when the block must stay dense.  `used`
+// (scratch, one byte per row of every job) marks the rows already pivoted.
 __global__ void __launch_bounds__(so::kThreads) so_aca_kernel(const SoAcaJob* __restrict__ jobs, int njobs,
                                                              const float* __restrict__ D, float* __restrict__ U,
                                                              float* __restrict__ V, unsigned char* __restrict__ used,
