@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(max_threads(MG, EV), 1) aca_block_kernel(Kerne
                     float* out = v + (int64_t)g0 * ldn + (sub.start - fb.col0);
                     for (int k = tid; k < ng * sub.size; k += nth) {
                         const int g = k / sub.size, j = k - g * sub.size;
-                        out[(int64_t)g * ldn + j] = sh.acc[j * MG + g] * P.cf[g0 + g];
+                        out[(int64_t)g * ldn + j] = times_c(P, sh.acc[j * MG + g], g0 + g);
                     }
                     __syncthreads();
                 }

@@ -547,6 +547,7 @@ int build(rt::Operator& op, const rt_problem* P, const rt_hparams* H, cudaStream
         const double l = -log2e * op.gc[g];
         kp.cl[g] = (float)l;
         kp.clo[g] = (float)(l - kp.cl[g]);
+        kp.cflo[g] = (float)(op.gc[g] - kp.cf[g]);
     }
     kp.wall_inside = kp.has_wall && inside_first_wall(kp, xyz64) ? 1 : 0;
     phase_setup(op, xyz64);

@@ -109,6 +109,7 @@ struct KernelParams {
     float olof[kMaxObst][3], ohif[kMaxObst][3];
     float dcl, dclo;           // -dc log2(e), -c_g log2(e): FP32 value and remainder
     float cl[kMaxGroups], clo[kMaxGroups];
+    float cflo[kMaxGroups];    // c_g - cf[g]
     const float4 *pxyz, *pcos; // [N] permuted coordinates, cosines
     const float4* tcen;        // [T] centroid, (2 diameters)^2
     const float4 *tpt, *tcos;  // [4][T] point and weight, cosines

@@ -67,6 +67,10 @@ __device__ __forceinline__ float group_exp(float hi, float lo, float tau, float 
     return ex2_approx(fmaf(hi, tau, fmaf(lo, tau, bias)));
 }
 
+// a finished sum times c_g.  c_g has a remainder as in the exponent: rounding it
+// here alone would shift every entry of the group one way (up to 6e-8).
+__device__ __forceinline__ float times_c(const KernelParams& P, float v, int g) { return fmaf(v, P.cf[g], v * P.cflo[g]); }
+
 // pairs of FP32 values in one 64-bit register: one instruction for two groups
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack2(float a, float b)

@@ -21,7 +21,10 @@
 //   box with grid, walls and corners, 1 group (EV_GENERAL): 901 -> 450 ms
 // Near blocks alone now: 66 ms (32^3), 80 ms (41^3, 98 before the point loops were
 // rolled up and six CTAs ran on an SM).
-// Error of a matvec against FP64, every block dense: 1.34e-7 before and after.
+// Error against the FP64 oracle, every block dense, before (positions, one group scale
+// in FP32 everywhere) and after: entries (root mean square) 1.37e-7 -> 1.33e-7, matvec
+// 9.8e-8 -> 9.3e-8 (10^3, 1 group, wall z = 0); 1.36e-7 -> 1.33e-7, 1.07e-7 -> 1.00e-7
+// (wall x = 1); 1.63e-7 -> 1.40e-7, 1.17e-7 -> 1.15e-7 (8^3, 16 groups).
 //
 // (tetrahedron, term) pairs whose source point is near (14-point rule) are
 // listed in shared memory and worked off with all lanes full.
@@ -513,12 +516,12 @@ __device__ __forceinline__ void column_chunk(const KernelParams& P, int row0, in
             if (g0 + g >= P.G) break;
             float v = 0.f;
             for (int k = 0; k < parts; ++k) v += sh.red[(k * mc + r) * MG + g];
-            out[(int64_t)(g0 + g) * gstride + r] = v * P.cf[g0 + g];
+            out[(int64_t)(g0 + g) * gstride + r] = times_c(P, v, g0 + g);
         }
     } else if (live) {
 #pragma unroll
         for (int g = 0; g < MG; ++g)
-            if (g0 + g < P.G) out[(int64_t)(g0 + g) * gstride + pos] = acc.get(g) * P.cf[g0 + g];
+            if (g0 + g < P.G) out[(int64_t)(g0 + g) * gstride + pos] = times_c(P, acc.get(g), g0 + g);
     }
     __syncthreads();
 }

@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(max_threads(MG, EV), 1) row_items_kernel(Kerne
     for (int e = threadIdx.x; e < per * ng; e += blockDim.x) {
         const int g = e / per, k = e - g * per;
         const int j = k / it.nrow, r = k - j * it.nrow;
-        out[it.out + r + (int64_t)(g0 + g) * it.gs + (int64_t)j * it.js] = sh.acc[((int64_t)r * n + j) * MG + g] * P.cf[g0 + g];
+        out[it.out + r + (int64_t)(g0 + g) * it.gs + (int64_t)j * it.js] = times_c(P, sh.acc[((int64_t)r * n + j) * MG + g], g0 + g);
     }
 }
 

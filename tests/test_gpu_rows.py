@@ -212,3 +212,28 @@ def test_equally_spaced_scales_in_either_order_at_large_depth(k0, c, wall):
                 size = np.linalg.norm(ref[g])
                 assert np.linalg.norm(got[g] - ref[g]) <= 7e-5 * size + 1e-30 * p.N, (g, size)
         op.free()
+
+
+@pytest.mark.parametrize("wall,kind", [(Z0, "sin"), (Z0, "const"), (OBLIQUE, "sin"), (Z0, "grid")])
+def test_entries_are_not_shifted_by_the_rounding_of_a_group_scale(wall, kind):
+    """Scales just below and just above the middle between two FP32 numbers round 5.8e-8 apart from their
+    values in opposite directions.  The mean relative error over all entries, in which every other
+    rounding is the same up to 1/sqrt(entries), may differ by 2e-8 between the two."""
+    import paper_2306_05789_gb300 as rt
+    from oracle import oracle as O
+    mean = []
+    for c in (1.0 + 0.49 * 2.0 ** -23, 1.0 + 0.51 * 2.0 ** -23):
+        p = _problem(7, 1, wall, kind)
+        p.freqs.c = np.array([c])
+        ref = O.DenseOperator(p)
+        op = rt.rt_build_operator(p, rt.hparams(eta=1e-9))
+        err = 0.0
+        for j in range(p.N):
+            x = np.zeros((1, p.N), dtype=np.float32)
+            x[0, j] = 1.0
+            col = ref.G[0][:, j]
+            rel = (_apply(op, x)[0] - col) / col
+            err += float(np.median(rel)) / p.N   # a column's middle: the grid's kinks have a long tail
+        mean.append(err)
+        op.free()
+    assert abs(mean[0] - mean[1]) < 2e-8, mean
