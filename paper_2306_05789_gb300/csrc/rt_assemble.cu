@@ -734,12 +734,16 @@ __global__ void __launch_bounds__(256) aca_pack(AcaDev D, const PackItem* items,
         if constexpr (sizeof(T) == 4) {
             const int64_t* toff = D.toff + (int64_t)p.b * D.rmax;
             const int tid = blockIdx.y * blockDim.x + threadIdx.x, nth = gridDim.y * blockDim.x;
+            // 32-bit counters over at most 2^30 elements at a time
             const int nq = n4 >> 2, per = D.G * nq;   // float4s of one term's V
+            for (int l0 = 0, lc; l0 < p.r; l0 += lc) {
+                lc = min(p.r - l0, max(1, (1 << 30) / per));
 #pragma unroll 4
-            for (int e = tid; e < p.r * per; e += nth) {
-                const int l = e / per, k = e - l * per, g = k / nq;
-                const float4 x = reinterpret_cast<const float4*>(D.pool + toff[l] + (int64_t)D.G * m4)[k];
-                *reinterpret_cast<float4*>(dst + p.voff_dst + ((int64_t)g * p.r + l) * n8 + 4 * (k - g * nq)) = x;
+                for (int e = tid; e < lc * per; e += nth) {
+                    const int lr = e / per, k = e - lr * per, g = k / nq, l = l0 + lr;
+                    const float4 x = reinterpret_cast<const float4*>(D.pool + toff[l] + (int64_t)D.G * m4)[k];
+                    *reinterpret_cast<float4*>(dst + p.voff_dst + ((int64_t)g * p.r + l) * n8 + 4 * (k - g * nq)) = x;
+                }
             }
             for (int c = p.c0; c < p.c1; ++c) {
                 const Chunk ch = chunks[c];
