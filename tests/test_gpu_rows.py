@@ -237,3 +237,24 @@ def test_entries_are_not_shifted_by_the_rounding_of_a_group_scale(wall, kind):
         mean.append(err)
         op.free()
     assert abs(mean[0] - mean[1]) < 2e-8, mean
+
+
+@pytest.mark.parametrize("groups", [1, 4, 5, 8, 9, 17])
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("kind", ["const", "sin", "grid"])
+def test_dense_matrix_of_every_group_chunk_matches_oracle(groups, prec, kind):
+    """Dense mode at the edges of its instances (1, 4, 8 and 16 groups a pass).  FP64: sums of positive
+    terms with about ten roundings each and a depth within 1e-14; FP32 as the rows above."""
+    import torch
+
+    import paper_2306_05789_gb300 as rt
+    from oracle import oracle as O
+    f64 = prec == "f64"
+    p = _problem(5, groups, Z0, kind)
+    X = W.rand_vectors((groups, p.N), seed=1)
+    X = X if f64 else X.astype(np.float32)
+    ref = O.DenseOperator(p).apply(X.astype(np.float64))
+    op = rt.rt_build_operator(p, rt.hparams(mode=rt.RT_MODE_DENSE, prec=rt.RT_PREC_F64 if f64 else rt.RT_PREC_F32))
+    got = _apply(op, X)
+    op.free()
+    assert np.linalg.norm(got - ref) < (1e-13 if f64 else 2e-6) * np.linalg.norm(ref)
