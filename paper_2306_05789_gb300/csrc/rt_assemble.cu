@@ -202,6 +202,23 @@ static int grid_for(int64_t warps)
 // ---------------------------------------------------------------------------
 // dense mode: the whole matrix [G][N][N] row-major
 // ---------------------------------------------------------------------------
+// A sum of many terms: FP32 compensated (Kahan), FP64 plain.  A sum that has
+// overflowed stays infinite: its compensation would be inf - inf.
+template <class R>
+struct Sum {
+    R v = R(0), lost = R(0);
+    __device__ __forceinline__ void add(R x)
+    {
+        if constexpr (sizeof(R) == 4) {
+            const R y = x - lost, t = v + y;
+            lost = isinf(t) ? R(0) : (t - v) - y;
+            v = t;
+        } else {
+            v += x;
+        }
+    }
+};
+
 // A thread takes one tetrahedron of one row and evaluates every point once for
 // the four hat functions of its vertices (entry by entry, each point was
 // evaluated four times); the vertex sums go to scratch [row][vertex slot][g][T]
@@ -215,22 +232,6 @@ static int grid_for(int64_t warps)
 // compensated (FP32).  Root mean square error of an entry against extended precision,
 // 5^3, oblique wall: FP64 2.03e-16 (entry evaluator 2.03e-16, serial sums 2.20e-16),
 // FP32 1.17e-7 (1.16e-7; serial sums, rsqrt and one weight a point 1.40e-7).
-// A sum of many terms: FP32 compensated (Kahan), FP64 plain
-template <class R>
-struct Sum {
-    R v = R(0), lost = R(0);
-    __device__ __forceinline__ void add(R x)
-    {
-        if constexpr (sizeof(R) == 4) {
-            const R y = x - lost, t = v + y;
-            lost = (t - v) - y;
-            v = t;
-        } else {
-            v += x;
-        }
-    }
-};
-
 constexpr int kDenseThreads = 128;
 template <class R, int MG, bool XT>
 __global__ void __launch_bounds__(kDenseThreads) dense_tets_kernel(KernelParams P, int row0, int g0, R* __restrict__ scratch)
@@ -376,7 +377,7 @@ static int dense_matrix(Operator& op, cudaStream_t s, std::string& err)
     op.d_dense = d;
     if (op.G <= 1) return dense_rows<R, 1>(op, d, s, err);
     if (op.G <= 4) return dense_rows<R, 4>(op, d, s, err);
-    if (op.G <= 8) return dense_rows<R, 8>(op, d, s, err);   // 11^3, 8 groups: FP32 4.4 -> 2.3 ms, FP64 47 -> 41 ms
+    if (op.G <= 8) return dense_rows<R, 8>(op, d, s, err);   // 11^3, 8 groups: FP32 4.4 -> 2.7 ms, FP64 47 -> 41 ms
     return dense_rows<R, 16>(op, d, s, err);
 }
 

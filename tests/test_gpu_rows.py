@@ -258,3 +258,16 @@ def test_dense_matrix_of_every_group_chunk_matches_oracle(groups, prec, kind):
     got = _apply(op, X)
     op.free()
     assert np.linalg.norm(got - ref) < (1e-13 if f64 else 2e-6) * np.linalg.norm(ref)
+
+
+def test_dense_sums_that_overflow_are_infinite():
+    """Cells of 2e13 units a side have volumes beyond FP32: the FP32 dense matrix is infinite throughout,
+    not NaN (positive terms only)."""
+    import paper_2306_05789_gb300 as rt
+    p = _problem(4, 2, Z0, "const")
+    p.xyz = p.xyz * 6e13
+    p.kappa.k0 = 1e-14
+    op = rt.rt_build_operator(p, rt.hparams(mode=rt.RT_MODE_DENSE, prec=rt.RT_PREC_F32))
+    got = _apply(op, np.ones((2, p.N), dtype=np.float32))
+    op.free()
+    assert np.isposinf(got).all()
